@@ -744,12 +744,13 @@ rsg_status orthonormalize_dev(rsg_ham H, void *psi, int64_t S, int64_t ld, doubl
     }
     if (H->dtype == RSG_C64) {
         // FP64 norms for the diagonal, FP32 runs summed in FP64 elsewhere
-        CK(H->Wc.ensure((size_t)S * S * 8 + (size_t)S * sizeof(double)));
-        double *nrm = (double *)((char *)H->Wc.p + (size_t)S * S * 8);
+        const size_t nrm_bytes = ((size_t)S * sizeof(double) + 255) / 256 * 256;
+        CK(H->Wc.ensure(nrm_bytes + tri_c64_bytes((int)S)));
+        double *nrm = H->Wc.as<double>();
         CKS(norms_dev(H, psi, S, ld, nrm, st));
         CK(launch_gram_c64(psi, P, (int)ld, (int)S, h3, H->red.as<double>(), nb, H->G.as<double>(), nrm, st));
         CK(launch_chol_inv(H->G.as<double>(), H->W.as<double>(), (int)S, drift_dev, H->status.as<int>(), st));
-        CK(launch_tri_apply_c64(psi, P, (int)ld, (int)S, H->W.as<double>(), H->Wc.p, st));
+        CK(launch_tri_apply_c64(psi, P, (int)ld, (int)S, H->W.as<double>(), (char *)H->Wc.p + nrm_bytes, st));
     } else {
         CK(launch_gram<double>(psi, P, (int)ld, (int)S, h3, H->red.as<double>(), nb, H->G.as<double>(), st));
         CK(launch_chol_inv(H->G.as<double>(), H->W.as<double>(), (int)S, drift_dev, H->status.as<int>(), st));

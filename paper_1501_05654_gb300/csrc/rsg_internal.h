@@ -153,7 +153,10 @@ cudaError_t launch_proj_reduce(const double *partial, int SV, const ProjDev &pj,
 template <typename R>
 cudaError_t launch_proj_scatter(const ApplyArgs<R> &a, const ProjDev &pj, cudaStream_t st);
 
-// ---- linear algebra on state blocks (rsg_linalg.cu) ----
+// ---- linear algebra on state blocks (rsg_linalg.cu, rsg_qr.cu) ----
+// out[i] = scale * sum over nblk rows of partial[b * n + i], in a fixed order.
+cudaError_t launch_sum_blocks(const double *partial, int nblk, int64_t n, double scale, double *out,
+                              cudaStream_t st);
 // G (S x S complex double) = h3 * Psi^H Phi (cross Gram; partial as launch_gram).
 template <typename R>
 cudaError_t launch_cross_gram(const void *psi, const void *phi, int64_t P, int ld, int S, double h3,
@@ -185,11 +188,16 @@ int gram_blocks(int64_t P, int S);
 // the diagonal is replaced by the given FP64 norms (h3 applied).
 cudaError_t launch_gram_c64(const void *psi, int64_t P, int ld, int S, double h3, double *partial,
                             int nblk, double *G, const double *norms, cudaStream_t st);
-// complex64 triangular update with W^H rounded to FP32 (Wc_buf: S*S float2).
-cudaError_t launch_tri_apply_c64(void *psi, int64_t P, int ld, int S, const double *W, void *Wc_buf,
+// complex64 triangular update with W^H rounded to FP32 (Wt_buf: tri_c64_bytes(S)
+// bytes, 16-byte aligned; may be NULL when that is 0).
+cudaError_t launch_tri_apply_c64(void *psi, int64_t P, int ld, int S, const double *W, void *Wt_buf,
                                  cudaStream_t st);
-// In-place Cholesky of G, inverse of the factor into W (S x S complex double),
-// drift[s] = max(drift[s], |G_ss - 1|), status word set non-zero on failure.
+size_t tri_c64_bytes(int S);
+cudaError_t launch_norms_c64(const void *psi, int64_t P, int ld, int S, double h3, double *partial, int nblk,
+                             double *out, cudaStream_t st);
+// Cholesky factor of G (G is overwritten), its inverse into W (S x S complex
+// double), drift[s] = max(drift[s], |G_ss - 1|), status word set non-zero on
+// failure.
 cudaError_t launch_chol_inv(double *G, double *W, int S, double *drift, int *status,
                             cudaStream_t st);
 // psi <- psi W^H (in place).

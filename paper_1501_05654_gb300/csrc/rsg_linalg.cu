@@ -4,7 +4,8 @@
 // inverse are kept in FP64 for both compute types (arXiv:1501.05654,
 // Sec. "Parallelization, optimizations and graphics processing units": real-time propagation preserves orthogonality, so the
 // states are re-orthonormalised only now and then; here Cholesky-QR, which
-// equals Gram-Schmidt in index order).  The adjoint inner products of the
+// equals Gram-Schmidt in index order; the Gram matrices, the factor and the
+// complex64 update are in rsg_qr.cu).  The adjoint inner products of the
 // control gradient (Sec. "Quantum optimal control", Eq. (qoctgradient)) are
 // FP64 reductions as well.
 #include "rsg_internal.h"
@@ -20,96 +21,7 @@ __device__ __forceinline__ void ld_c(const R *p, double &re, double &im) {
     im = (double)p[1];
 }
 
-constexpr int GT = 16;   // Gram tile edge
-
 }  // namespace
-
-int gram_blocks(int64_t P, int S) {
-    (void)S;
-    int64_t n = (P + 4095) / 4096;
-    if (n > 296) n = 296;
-    if (n < 1) n = 1;
-    return (int)n;
-}
-
-int norm_blocks(int64_t P) {
-    int64_t n = (P + 2047) / 2048;
-    if (n > 608) n = 608;
-    if (n < 1) n = 1;
-    return (int)n;
-}
-
-// partial[blk][s][t] (complex double) = sum over the block's points of
-// conj(psi[p,s]) phi[p,t] for one GT x GT tile of (s, t) (phi = psi: the Gram
-// matrix; phi = H psi: the Rayleigh-Ritz matrix of the eigensolver).
-template <typename R>
-__global__ void __launch_bounds__(GT *GT) k_gram(const R *__restrict__ psi, const R *__restrict__ phi, int64_t P,
-                                                 int ld, int S, double *__restrict__ partial, int nblk) {
-    __shared__ double sa[GT][GT][2], sb[GT][GT][2];
-    const int s0 = blockIdx.x * GT, t0 = blockIdx.y * GT;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int64_t per = (P + nblk - 1) / nblk;
-    const int64_t p0 = blockIdx.z * per;
-    const int64_t p1 = p0 + per < P ? p0 + per : P;
-    double gr = 0.0, gi = 0.0;
-    for (int64_t pb = p0; pb < p1; pb += GT) {
-        // stage GT points x GT columns of both tiles
-        const int64_t p = pb + ty;
-        double ar = 0, ai = 0, br = 0, bi = 0;
-        if (p < p1) {
-            if (s0 + tx < S) ld_c(psi + (p * ld + s0 + tx) * 2, ar, ai);
-            if (t0 + tx < S) ld_c(phi + (p * ld + t0 + tx) * 2, br, bi);
-        }
-        sa[ty][tx][0] = ar;
-        sa[ty][tx][1] = ai;
-        sb[ty][tx][0] = br;
-        sb[ty][tx][1] = bi;
-        __syncthreads();
-#pragma unroll 4
-        for (int k = 0; k < GT; k++) {
-            const double xr = sa[k][ty][0], xi = sa[k][ty][1];   // psi[p, s0+ty]
-            const double yr = sb[k][tx][0], yi = sb[k][tx][1];   // psi[p, t0+tx]
-            gr += xr * yr + xi * yi;
-            gi += xr * yi - xi * yr;
-        }
-        __syncthreads();
-    }
-    const int s = s0 + ty, t = t0 + tx;
-    if (s < S && t < S) {
-        double *d = partial + (((int64_t)blockIdx.z * S + s) * S + t) * 2;
-        d[0] = gr;
-        d[1] = gi;
-    }
-}
-
-__global__ void k_sum_blocks(const double *__restrict__ partial, int nblk, int64_t n, double scale,
-                             double *__restrict__ out) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double s = 0.0;
-    for (int b = 0; b < nblk; b++) s += partial[(int64_t)b * n + i];
-    out[i] = scale * s;
-}
-
-template <typename R>
-cudaError_t launch_gram(const void *psi, int64_t P, int ld, int S, double h3, double *partial,
-                        int nblk, double *G, cudaStream_t st) {
-    dim3 grid((S + GT - 1) / GT, (S + GT - 1) / GT, nblk);
-    k_gram<R><<<grid, dim3(GT, GT), 0, st>>>((const R *)psi, (const R *)psi, P, ld, S, partial, nblk);
-    const int64_t n = (int64_t)S * S * 2;
-    k_sum_blocks<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(partial, nblk, n, h3, G);
-    return cudaGetLastError();
-}
-
-template <typename R>
-cudaError_t launch_cross_gram(const void *psi, const void *phi, int64_t P, int ld, int S, double h3,
-                              double *partial, int nblk, double *G, cudaStream_t st) {
-    dim3 grid((S + GT - 1) / GT, (S + GT - 1) / GT, nblk);
-    k_gram<R><<<grid, dim3(GT, GT), 0, st>>>((const R *)psi, (const R *)phi, P, ld, S, partial, nblk);
-    const int64_t n = (int64_t)S * S * 2;
-    k_sum_blocks<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(partial, nblk, n, h3, G);
-    return cudaGetLastError();
-}
 
 // psi[p, s] <- sum_t psi[p, t] Q[t][s] (Q: S x S complex double, the Ritz
 // rotation), in place: each block stages its full rows in shared memory.
@@ -223,8 +135,7 @@ template <typename R>
 cudaError_t launch_bilinear(const void *x, const void *y, int64_t P, int ld, int S, double h3, double *partial,
                             int nblk, double *out, cudaStream_t st) {
     k_bilinear<R><<<dim3(nblk, S), 256, 0, st>>>((const R *)x, (const R *)y, P, ld, S, partial, nblk);
-    k_sum_blocks<<<(unsigned)((2 * S + 255) / 256), 256, 0, st>>>(partial, nblk, 2 * (int64_t)S, h3, out);
-    return cudaGetLastError();
+    return launch_sum_blocks(partial, nblk, 2 * (int64_t)S, h3, out, st);
 }
 
 // z[p,s] = a[s] x[p,s] + b[s] y[p,s] with complex per-state a, b (device,
@@ -276,219 +187,7 @@ template <typename R>
 cudaError_t launch_resid(const void *x, const void *hx, int64_t P, int ld, int S, const double *lam, double h3,
                          double *partial, int nblk, double *out, cudaStream_t st) {
     k_resid<R><<<dim3(nblk, S), 256, 0, st>>>((const R *)x, (const R *)hx, P, ld, S, lam, partial, nblk);
-    k_sum_blocks<<<(unsigned)((S + 255) / 256), 256, 0, st>>>(partial, nblk, S, h3, out);
-    return cudaGetLastError();
-}
-
-// complex64 Gram matrix: FP32 products summed in FP32 over runs of 8 points,
-// runs summed in FP64.  Tile 32 x 32 of (s, t) per block, 2 x 2 entries per
-// thread (16 x 16 threads); partial[blk][s][t] as in k_gram.
-constexpr int G32 = 32, GRUN = 8;
-__global__ void __launch_bounds__(256) k_gram32(const float2 *__restrict__ psi, int64_t P, int ld, int S,
-                                                double *__restrict__ partial, int nblk) {
-    __shared__ float2 sa[GRUN][G32], sb[GRUN][G32];
-    const int s0 = blockIdx.x * G32, t0 = blockIdx.y * G32;
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 16 + tx;
-    const int64_t per = (P + nblk - 1) / nblk;
-    const int64_t p0 = blockIdx.z * per;
-    const int64_t p1 = p0 + per < P ? p0 + per : P;
-    double ar[2][2] = {{0, 0}, {0, 0}}, ai[2][2] = {{0, 0}, {0, 0}};
-    for (int64_t pb = p0; pb < p1; pb += GRUN) {
-        // stage GRUN points x 32 columns of both tiles (256 threads, one value each)
-        {
-            const int q = tid / G32, col = tid % G32;
-            const int64_t p = pb + q;
-            float2 va = make_float2(0.f, 0.f), vb = make_float2(0.f, 0.f);
-            if (p < p1) {
-                if (s0 + col < S) va = psi[p * ld + s0 + col];
-                if (t0 + col < S) vb = psi[p * ld + t0 + col];
-            }
-            sa[q][col] = va;
-            sb[q][col] = vb;
-        }
-        __syncthreads();
-        float fr[2][2] = {{0, 0}, {0, 0}}, fi[2][2] = {{0, 0}, {0, 0}};
-#pragma unroll
-        for (int k = 0; k < GRUN; k++) {
-            const float2 x0 = sa[k][ty], x1 = sa[k][ty + 16];   // psi[p, s]
-            const float2 y0 = sb[k][tx], y1 = sb[k][tx + 16];   // psi[p, t]
-            const float2 xs[2] = {x0, x1}, ys[2] = {y0, y1};
-#pragma unroll
-            for (int a = 0; a < 2; a++)
-#pragma unroll
-                for (int b = 0; b < 2; b++) {
-                    // conj(x) y
-                    fr[a][b] = fmaf(xs[a].x, ys[b].x, fmaf(xs[a].y, ys[b].y, fr[a][b]));
-                    fi[a][b] = fmaf(xs[a].x, ys[b].y, fmaf(-xs[a].y, ys[b].x, fi[a][b]));
-                }
-        }
-#pragma unroll
-        for (int a = 0; a < 2; a++)
-#pragma unroll
-            for (int b = 0; b < 2; b++) {
-                ar[a][b] += (double)fr[a][b];
-                ai[a][b] += (double)fi[a][b];
-            }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 2; a++)
-#pragma unroll
-        for (int b = 0; b < 2; b++) {
-            const int s = s0 + ty + 16 * a, t = t0 + tx + 16 * b;
-            if (s < S && t < S) {
-                double *d = partial + (((int64_t)blockIdx.z * S + s) * S + t) * 2;
-                d[0] = ar[a][b];
-                d[1] = ai[a][b];
-            }
-        }
-}
-
-// Replace the Gram diagonal with FP64 norms (h3 already applied to both).
-__global__ void k_set_diag(double *G, const double *norms, int S) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= S) return;
-    G[((int64_t)s * S + s) * 2] = norms[s];
-    G[((int64_t)s * S + s) * 2 + 1] = 0.0;
-}
-
-cudaError_t launch_gram_c64(const void *psi, int64_t P, int ld, int S, double h3, double *partial, int nblk,
-                            double *G, const double *norms, cudaStream_t st) {
-    dim3 grid((S + G32 - 1) / G32, (S + G32 - 1) / G32, nblk);
-    k_gram32<<<grid, dim3(16, 16), 0, st>>>((const float2 *)psi, P, ld, S, partial, nblk);
-    const int64_t n = (int64_t)S * S * 2;
-    k_sum_blocks<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(partial, nblk, n, h3, G);
-    k_set_diag<<<(S + 127) / 128, 128, 0, st>>>(G, norms, S);
-    return cudaGetLastError();
-}
-
-// complex64 triangular update psi[p, s] <- sum_{t <= s} psi[p, t] conj(W[s][t])
-// with W rounded to FP32 (the states are FP32): rows staged in shared
-// memory (in place), W^H read from global (L1/L2 resident).
-__global__ void k_wconj32(const double *__restrict__ W, float2 *__restrict__ Wc, int S) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S * S) return;
-    Wc[i] = make_float2((float)W[2 * i], (float)-W[2 * i + 1]);
-}
-
-__global__ void __launch_bounds__(256) k_tri_apply32(float2 *psi, int64_t P, int ld, int S,
-                                                     const float2 *__restrict__ Wc, int pt) {
-    extern __shared__ float2 rows[];   // pt x S
-    const int64_t p0 = (int64_t)blockIdx.x * pt;
-    const int n = pt * S;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int q = e / S, t = e - q * S;
-        const int64_t p = p0 + q;
-        rows[e] = p < P ? psi[p * ld + t] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int s = e % S, q = e / S;
-        const int64_t p = p0 + q;
-        if (p >= P) continue;
-        const float2 *row = rows + q * S;
-        const float2 *w = Wc + (int64_t)s * S;
-        float re = 0.f, im = 0.f;
-        for (int t = 0; t <= s; t++) {
-            const float2 a = row[t], b = w[t];
-            re = fmaf(a.x, b.x, fmaf(-a.y, b.y, re));
-            im = fmaf(a.x, b.y, fmaf(a.y, b.x, im));
-        }
-        psi[p * ld + s] = make_float2(re, im);
-    }
-}
-
-cudaError_t launch_tri_apply_c64(void *psi, int64_t P, int ld, int S, const double *W, void *Wc_buf,
-                                 cudaStream_t st) {
-    k_wconj32<<<(S * S + 255) / 256, 256, 0, st>>>(W, (float2 *)Wc_buf, S);
-    int pt = 8192 / S;
-    if (pt < 1) pt = 1;
-    if (pt > 128) pt = 128;
-    const size_t smem = (size_t)pt * S * sizeof(float2);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_tri_apply32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    const int64_t nb = (P + pt - 1) / pt;
-    k_tri_apply32<<<(unsigned)nb, 256, smem, st>>>((float2 *)psi, P, ld, S, (const float2 *)Wc_buf, pt);
-    return cudaGetLastError();
-}
-
-// One block.  G (S x S complex double, G[i][j] = <psi_i|psi_j>) is factored
-// in place as G = L L^H (lower L); W = L^-1.  drift (optional) records
-// |G_ss - 1|.  status != 0 if G is not finite or not positive definite.
-__global__ void k_chol_inv(double *G, double *W, int S, double *drift, int *status) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    __shared__ int bad;
-    if (tid == 0) bad = 0;
-    __syncthreads();
-    for (int s = tid; s < S; s += nt) {
-        const double d = G[((int64_t)s * S + s) * 2];
-        if (drift != nullptr) {
-            const double e = fabs(d - 1.0);
-            if (!(e <= drift[s])) drift[s] = e;   // NaN propagates
-        }
-    }
-    for (int64_t i = tid; i < (int64_t)S * S * 2; i += nt)
-        if (!isfinite(G[i])) bad = 1;
-    __syncthreads();
-    for (int j = 0; j < S && !bad; j++) {
-        if (tid == 0) {
-            double d = G[((int64_t)j * S + j) * 2];
-            for (int k = 0; k < j; k++) {
-                const double *l = G + ((int64_t)j * S + k) * 2;
-                d -= l[0] * l[0] + l[1] * l[1];
-            }
-            if (!(d > 0.0)) bad = 1;
-            G[((int64_t)j * S + j) * 2] = d > 0.0 ? sqrt(d) : 1.0;
-            G[((int64_t)j * S + j) * 2 + 1] = 0.0;
-        }
-        __syncthreads();
-        const double ljj = G[((int64_t)j * S + j) * 2];
-        for (int i = j + 1 + tid; i < S; i += nt) {
-            // L[i][j] = (G[i][j] - sum_k L[i][k] conj(L[j][k])) / L[j][j]
-            double re = G[((int64_t)i * S + j) * 2], im = G[((int64_t)i * S + j) * 2 + 1];
-            for (int k = 0; k < j; k++) {
-                const double *a = G + ((int64_t)i * S + k) * 2;
-                const double *b = G + ((int64_t)j * S + k) * 2;
-                re -= a[0] * b[0] + a[1] * b[1];
-                im -= a[1] * b[0] - a[0] * b[1];
-            }
-            G[((int64_t)i * S + j) * 2] = re / ljj;
-            G[((int64_t)i * S + j) * 2 + 1] = im / ljj;
-        }
-        __syncthreads();
-    }
-    if (bad) {
-        if (tid == 0) *status = 1;
-        return;
-    }
-    // W = L^-1, one column per thread (forward substitution)
-    for (int c = tid; c < S; c += nt) {
-        for (int i = 0; i < S; i++) {
-            W[((int64_t)i * S + c) * 2] = 0.0;
-            W[((int64_t)i * S + c) * 2 + 1] = 0.0;
-        }
-        W[((int64_t)c * S + c) * 2] = 1.0 / G[((int64_t)c * S + c) * 2];
-        for (int i = c + 1; i < S; i++) {
-            double re = 0.0, im = 0.0;
-            for (int k = c; k < i; k++) {
-                const double *l = G + ((int64_t)i * S + k) * 2;
-                const double *w = W + ((int64_t)k * S + c) * 2;
-                re += l[0] * w[0] - l[1] * w[1];
-                im += l[0] * w[1] + l[1] * w[0];
-            }
-            const double lii = G[((int64_t)i * S + i) * 2];
-            W[((int64_t)i * S + c) * 2] = -re / lii;
-            W[((int64_t)i * S + c) * 2 + 1] = -im / lii;
-        }
-    }
-}
-
-cudaError_t launch_chol_inv(double *G, double *W, int S, double *drift, int *status,
-                            cudaStream_t st) {
-    k_chol_inv<<<1, 256, 0, st>>>(G, W, S, drift, status);
-    return cudaGetLastError();
+    return launch_sum_blocks(partial, nblk, S, h3, out, st);
 }
 
 // psi[p, s] <- sum_{t <= s} psi[p, t] conj(W[s][t]); each block stages its
@@ -572,10 +271,10 @@ __global__ void __launch_bounds__(256) k_norms(const R *__restrict__ psi, int64_
 template <typename R>
 cudaError_t launch_norms(const void *psi, int64_t P, int ld, int S, double h3, double *partial,
                          int nblk, double *out, cudaStream_t st) {
+    if constexpr (sizeof(R) == 4) return launch_norms_c64(psi, P, ld, S, h3, partial, nblk, out, st);
     const int bx = S < 32 ? S : 32;
     k_norms<R><<<nblk, dim3(bx, 256 / bx), 0, st>>>((const R *)psi, P, ld, S, partial, nblk);
-    k_sum_blocks<<<(S + 255) / 256, 256, 0, st>>>(partial, nblk, S, h3, out);
-    return cudaGetLastError();
+    return launch_sum_blocks(partial, nblk, S, h3, out, st);
 }
 
 // Ten inner products <b_j| X |a_i>, j + i <= 3, for the adjoint gradient.
@@ -737,7 +436,7 @@ cudaError_t launch_adjoint_dots(const void *const *b, const void *const *a, int6
                                              (const R *)a[2], (const R *)a[3], P, ld, X, partial,
                                              nblk);
     double *packed = partial + (int64_t)nblk * 20;
-    k_sum_blocks<<<1, 32, 0, st>>>(partial, nblk, 20, h3, packed);
+    if (cudaError_t e = launch_sum_blocks(partial, nblk, 20, h3, packed, st)) return e;
     k_adjoint_finish<<<1, 32, 0, st>>>(packed, out);
     return cudaGetLastError();
 }
@@ -779,8 +478,7 @@ template <typename R>
 cudaError_t launch_overlap(const void *f, const void *g, int64_t P, int ld, double h3,
                            double *partial, int nblk, double *out, cudaStream_t st) {
     k_overlap<R><<<nblk, 256, 0, st>>>((const R *)f, (const R *)g, P, ld, partial, nblk);
-    k_sum_blocks<<<1, 32, 0, st>>>(partial, nblk, 2, h3, out);
-    return cudaGetLastError();
+    return launch_sum_blocks(partial, nblk, 2, h3, out, st);
 }
 
 // y = a x + b y over n complex values
@@ -848,10 +546,6 @@ cudaError_t launch_grad_accum(const double *M, double tau, double *grad_k, cudaS
 }
 
 #define RSG_INST(R)                                                                               \
-    template cudaError_t launch_gram<R>(const void *, int64_t, int, int, double, double *, int,      \
-                                        double *, cudaStream_t);                                     \
-    template cudaError_t launch_cross_gram<R>(const void *, const void *, int64_t, int, int, double, \
-                                              double *, int, double *, cudaStream_t);                \
     template cudaError_t launch_rotate<R>(void *, int64_t, int, int, const double *, cudaStream_t);  \
     template cudaError_t launch_resid<R>(const void *, const void *, int64_t, int, int, const double *, \
                                          double, double *, int, double *, cudaStream_t);             \
