@@ -31,9 +31,8 @@ __device__ __forceinline__ ApplyArgs<float> batch_args(const SysArgs &S, int in_
     a.bi = 0.f;
     a.gr = a.gi = 0.f;
     a.nl_ptr = nullptr;
-    a.nl_ent = nullptr;
-    a.q_atom = nullptr;
-    a.q_p = nullptr;
+    a.e_atom = nullptr;
+    a.e_p = nullptr;
     a.D = nullptr;
     a.npmax = 0;
     a.P = S.P;

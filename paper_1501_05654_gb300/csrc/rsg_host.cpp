@@ -512,10 +512,13 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
     a.bi = (R)ep.bi;
     a.gr = (R)ep.gr;
     a.gi = (R)ep.gi;
+    a.ef = (a.fx != 0 || a.fy != 0 || a.fz != 0 ? EF_FIELD : 0) | (a.f0 != 0 ? EF_SHIFT : 0) |
+           (ep.ar == 0 && (!ep.twocol || ep.ar1 == 0) ? EF_IMAG : 0) |
+           (ep.ai == 0 && (!ep.twocol || ep.ai1 == 0) ? EF_REAL : 0) | (ep.br == 1 && ep.bi == 0 ? EF_BASE1 : 0) |
+           (ep.bi == 0 ? EF_BASER : 0) | (ep.gi == 0 ? EF_GAMR : 0);
     a.nl_ptr = H->pj.natoms > 0 ? H->pj.nl_ptr : nullptr;
-    a.nl_ent = H->pj.nl_ent;
-    a.q_atom = H->pj.q_atom;
-    a.q_p = (const R *)H->pj.q_p;
+    a.e_atom = H->pj.e_atom;
+    a.e_p = (const R *)H->pj.e_p;
     a.D = H->D.p;
     a.npmax = H->pj.npmax;
     a.P = m->P;

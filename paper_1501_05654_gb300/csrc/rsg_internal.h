@@ -41,6 +41,17 @@ struct TileCfg {
     int threads = 256;   // staged kernel: threads per block (256 with two blocks per SM, or 512)
 };
 
+// Facts about an application that its FP64 epilogue uses (ApplyArgs::ef).
+enum {
+    EF_FIELD = 1,    // fx, fy or fz nonzero
+    EF_SHIFT = 2,    // f0 nonzero
+    EF_IMAG = 4,     // ar = 0 (every column)
+    EF_REAL = 8,     // ai = 0 (every column)
+    EF_BASE1 = 16,   // base scale 1
+    EF_BASER = 32,   // base scale real
+    EF_GAMR = 64,    // gamma real
+};
+
 // Everything one H application needs, by value.  Pointers to the state
 // blocks are typed as the 16-byte vector of the compute type (float4 = two
 // complex64 values, double2 = one complex128 value).
@@ -61,13 +72,13 @@ struct ApplyArgs {
     R ar, ai, br, bi, gr, gi;
     // non-local part (may be absent: nl_ptr == nullptr)
     const int32_t *nl_ptr;   // P+1 CSR over points
-    const int32_t *nl_ent;   // global sphere-entry index q
-    const int32_t *q_atom;   // atom of each entry
-    const R *q_p;            // entry-major projector values (npmax per entry)
+    const int32_t *e_atom;   // per point-CSR entry: its atom
+    const R *e_p;            // per point-CSR entry: its npmax projector values
     const void *D;           // (natoms*npmax, SV) vectors: h_a <p|u>
     int npmax;
     int64_t P;
     int *err;                // device status word (bounded waits record timeouts)
+    int ef = 0;              // EF_* (set for complex128)
     // complex scaling in the register-blocked kernel: the complex diagonal
     // v_theta e^{2i theta} per point (interleaved); the caller folds the
     // kinetic rotation e^{-2i theta} into (ar, ai); nullptr otherwise

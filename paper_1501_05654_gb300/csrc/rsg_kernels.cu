@@ -20,8 +20,9 @@
 //                   nine z-neighbours in registers; x/y neighbours come
 //                   through L1.  Projector terms are added in the epilogue
 //                   through a per-point CSR list of sphere entries.
-//   k_apply_naive   one thread per (point, vector), all 25 neighbours loaded;
-//                   the plain reference GPU path.
+//   k_apply_naive   the plain GPU path: a thread per column of (point,
+//                   vector) marching along z (complex64); k_apply_row64 a
+//                   thread per (point, vector) (complex128).
 //   k_proj_dot      partial sums of <p_ai|u_s> over sphere chunks (FP32
 //                   products and partial sums for complex64, FP64 across
 //                   chunks), k_proj_reduce: h^3 sum over chunks, times h_a.
@@ -35,12 +36,41 @@
 
 namespace rsg {
 
+// Projector entries of one point: their range, and the atom of the first
+// (read ahead of use: pointer, atom, coefficients is a chain of three loads).
+struct NlPoint {
+    int e0, e1, at;
+};
+// acc += sum over the point's entries of p_ai D_ai, entries in list order.
+template <typename R>
+__device__ __forceinline__ void add_projectors(const ApplyArgs<R> &a, const NlPoint &n, int v,
+                                               typename VT<R>::T &acc) {
+    using T = typename VT<R>::T;
+    for (int e = n.e0; e < n.e1; e++) {
+        const int at = e == n.e0 ? n.at : a.e_atom[e];
+        const R *pv = a.e_p + (int64_t)e * a.npmax;
+        const T *Da = (const T *)a.D + (int64_t)at * a.npmax * a.SV + v;
+        for (int i = 0; i < a.npmax; i++) VT<R>::fma(acc, pv[i], Da[(int64_t)i * a.SV]);
+    }
+}
+template <typename R>
+__device__ __forceinline__ NlPoint load_projectors(const ApplyArgs<R> &a, int64_t idx) {
+    NlPoint n{0, 0, 0};
+    if (a.nl_ptr != nullptr) {
+        n.e0 = a.nl_ptr[idx];
+        n.e1 = a.nl_ptr[idx + 1];
+        if (n.e0 < n.e1) n.at = a.e_atom[n.e0];
+    }
+    return n;
+}
+
 // ------------------------------------------------------------ epilogue ---
 template <typename R>
 __device__ __forceinline__ void finish_point(const ApplyArgs<R> &a, int64_t idx, int x, int y,
                                              int z, int v,
                                              const typename VT<R>::T &center,
-                                             typename VT<R>::T acc) {
+                                             typename VT<R>::T acc, R vloc,
+                                             const typename VT<R>::T &bval, const NlPoint &nl) {
     using V = VT<R>;
     using T = typename V::T;
     const int SV = a.SV;
@@ -48,7 +78,7 @@ __device__ __forceinline__ void finish_point(const ApplyArgs<R> &a, int64_t idx,
         // two columns with their own field terms: column (v, component
         // pair) of a complex64 vector, or vector v of complex128
         auto diag_of = [&](int c) {
-            return a.V[idx] + a.cf[c][0] + a.cf[c][1] * (R)x + a.cf[c][2] * (R)y + a.cf[c][3] * (R)z;
+            return vloc + a.cf[c][0] + a.cf[c][1] * (R)x + a.cf[c][2] * (R)y + a.cf[c][3] * (R)z;
         };
         if constexpr (sizeof(R) == 4) {
             const R d0 = diag_of(0), d1 = diag_of(1);
@@ -60,20 +90,10 @@ __device__ __forceinline__ void finish_point(const ApplyArgs<R> &a, int64_t idx,
             V::fma(acc, diag_of(v), center);
         }
     } else {
-        const R diag = a.V[idx] + a.f0 + a.fx * (R)x + a.fy * (R)y + a.fz * (R)z;
+        const R diag = vloc + a.f0 + a.fx * (R)x + a.fy * (R)y + a.fz * (R)z;
         V::fma(acc, diag, center);
     }
-    if (a.nl_ptr != nullptr) {
-        const int e0 = a.nl_ptr[idx], e1 = a.nl_ptr[idx + 1];
-        const T *D = (const T *)a.D;
-        for (int e = e0; e < e1; e++) {
-            const int q = a.nl_ent[e];
-            const int at = a.q_atom[q];
-            const R *pv = a.q_p + (int64_t)q * a.npmax;
-            const T *Da = D + (int64_t)at * a.npmax * SV + v;
-            for (int i = 0; i < a.npmax; i++) V::fma(acc, pv[i], Da[(int64_t)i * SV]);
-        }
-    }
+    add_projectors<R>(a, nl, v, acc);
     const int64_t o = idx * SV + v;
     T y0;
     if (a.twocol) {
@@ -87,13 +107,22 @@ __device__ __forceinline__ void finish_point(const ApplyArgs<R> &a, int64_t idx,
     } else {
         y0 = V::cmul(a.ar, a.ai, acc);
     }
-    if (a.base != nullptr) V::cfma(y0, a.br, a.bi, ((const T *)a.base)[o]);
+    if (a.base != nullptr) V::cfma(y0, a.br, a.bi, bval);
     ((T *)a.out)[o] = y0;
     if (a.acc != nullptr) {
         T s = a.acc_base != nullptr ? ((const T *)a.acc_base)[o] : ((T *)a.acc)[o];
         V::cfma(s, a.gr, a.gi, y0);
         ((T *)a.acc)[o] = s;
     }
+}
+
+// finish_point with the potential and the base value loaded here.
+template <typename R>
+__device__ __forceinline__ void finish_point(const ApplyArgs<R> &a, int64_t idx, int x, int y, int z, int v,
+                                             const typename VT<R>::T &center, typename VT<R>::T acc) {
+    using T = typename VT<R>::T;
+    const T b = a.base != nullptr ? ((const T *)a.base)[idx * a.SV + v] : VT<R>::zero();
+    finish_point<R>(a, idx, x, y, z, v, center, acc, a.V[idx], b, load_projectors<R>(a, idx));
 }
 
 // Value of vector v at bbox (x, row) or zero outside the mesh.
@@ -505,33 +534,236 @@ __global__ void __launch_bounds__(NT, MINB) k_apply_staged(const ApplyArgs<R> a,
 
 
 // --------------------------------------------------------------- naive ---
+// FP64 epilogue of k_apply_naive: the general one costs 20 FP64 instructions
+// a value, which the FP64 pipe (two a clock per SM) pays next to the 50 of
+// the stencil.  The host's flags (ApplyArgs::ef) name the terms that are
+// absent or whose scale is purely real or imaginary, and those cost nothing.
+__device__ __forceinline__ void finish_fp64(const ApplyArgs<double> &a, int64_t idx, int x, int y, int z, int v,
+                                            const double2 &c, double2 acc, double d, const double2 &b,
+                                            const NlPoint &nl) {
+    const int SV = a.SV, ef = a.ef;
+    if (a.twocol)
+        d += a.cf[v][0] + a.cf[v][1] * (double)x + a.cf[v][2] * (double)y + a.cf[v][3] * (double)z;
+    else if (ef & EF_FIELD)
+        d += a.f0 + a.fx * (double)x + a.fy * (double)y + a.fz * (double)z;
+    else if (ef & EF_SHIFT)
+        d += a.f0;
+    acc.x = fma(d, c.x, acc.x);
+    acc.y = fma(d, c.y, acc.y);
+    add_projectors<double>(a, nl, v, acc);
+    const int64_t o = idx * SV + v;
+    const double ar = a.twocol ? a.ca[v][0] : a.ar, ai = a.twocol ? a.ca[v][1] : a.ai;
+    double2 y0 = b;   // base scale 1, or no base (b = 0)
+    if (a.base != nullptr && !(ef & EF_BASE1))
+        y0 = ef & EF_BASER ? make_double2(a.br * b.x, a.br * b.y) : VT<double>::cmul(a.br, a.bi, b);
+    if (ef & EF_IMAG) {
+        y0.x = fma(-ai, acc.y, y0.x);
+        y0.y = fma(ai, acc.x, y0.y);
+    } else if (ef & EF_REAL) {
+        y0.x = fma(ar, acc.x, y0.x);
+        y0.y = fma(ar, acc.y, y0.y);
+    } else {
+        VT<double>::cfma(y0, ar, ai, acc);
+    }
+    ((double2 *)a.out)[o] = y0;
+    if (a.acc != nullptr) {
+        double2 s = a.acc_base != nullptr ? ((const double2 *)a.acc_base)[o] : ((double2 *)a.acc)[o];
+        if (ef & EF_GAMR) {
+            s.x = fma(a.gr, y0.x, s.x);
+            s.y = fma(a.gr, y0.y, s.y);
+        } else {
+            VT<double>::cfma(s, a.gr, a.gi, y0);
+        }
+        ((double2 *)a.acc)[o] = s;
+    }
+}
+
+// complex128 form of the plain kernel: one thread per (point, vector), all 24
+// neighbours loaded at once through L1.  A block lies in one (y, z) row, so
+// the 16 neighbour rows are looked up once per block.  Bound by the FP64 pipe
+// (56 instructions a value with the Horner epilogue, two a clock per SM:
+// 1.39 ms for 904,089 points x 16 states; measured 1.62 ms, 2.04 ms when every
+// thread looked up its rows and ran the general epilogue).  The z-march of
+// the complex64 form below reads less but leaves SMs idle at the end of a
+// launch (64^3 x 2 columns: 82 us against 60 us here).
+constexpr int kRowNT = 128;
 template <typename R>
-__global__ void __launch_bounds__(256) k_apply_naive(const ApplyArgs<R> a) {
-    using V = VT<R>;
-    using T = typename V::T;
+__global__ void __launch_bounds__(kRowNT, 4) k_apply_row64(const ApplyArgs<R> a) {
+    static_assert(sizeof(R) == 8, "complex128");
+    using V = VT<double>;
+    __shared__ int4 nr[16];   // rows y-1, y+1, z-1, z+1, y-2, ...: start - xmin, xmin, xmax
     const int row = blockIdx.x;
-    const int ny = a.ny, nz = a.nz, SV = a.SV;
-    const int y = row % ny, z = row / ny;
+    const int ny = a.ny, SV = a.SV;
     const Row rc = a.rows[row];
-    if (rc.xmin > rc.xmax) return;
-    const T *__restrict__ in = (const T *)a.in;
     const int n = (rc.xmax - rc.xmin + 1) * SV;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    if ((int)blockIdx.y * kRowNT >= n) return;
+    const int z = row / ny, y = row - z * ny;
+    if (threadIdx.x < 16) {
+        const int k = (threadIdx.x >> 2) + 1, sgn = threadIdx.x & 1 ? k : -k;
+        const Row r = threadIdx.x & 2 ? load_row(a.rows, y, z + sgn, ny, a.nz) : load_row(a.rows, y + sgn, z, ny, a.nz);
+        nr[threadIdx.x] = make_int4(r.start - r.xmin, r.xmin, r.xmax, 0);
+    }
+    __syncthreads();
+    const double2 *__restrict__ in = (const double2 *)a.in;
+    for (int t = blockIdx.y * kRowNT + threadIdx.x; t < n; t += gridDim.y * kRowNT) {
         const int xo = t / SV, v = t - xo * SV;
         const int x = rc.xmin + xo;
         const int64_t idx = (int64_t)rc.start + xo;
-        const T c = V::ldg(in + idx * SV + v);
-        T acc = V::scale((R)3 * a.w[0], c);
+        const NlPoint nl = load_projectors<double>(a, idx);
+        const double2 *own = in + idx * SV + v;
+        const double2 c = V::ldg(own);
+        double2 val[4][6];
+#pragma unroll
         for (int k = 1; k <= 4; k++) {
-            T s = V::add(row_value<R>(in, rc, x - k, SV, v), row_value<R>(in, rc, x + k, SV, v));
-            s = V::add(s, row_value<R>(in, load_row(a.rows, y - k, z, ny, nz), x, SV, v));
-            s = V::add(s, row_value<R>(in, load_row(a.rows, y + k, z, ny, nz), x, SV, v));
-            s = V::add(s, row_value<R>(in, load_row(a.rows, y, z - k, ny, nz), x, SV, v));
-            s = V::add(s, row_value<R>(in, load_row(a.rows, y, z + k, ny, nz), x, SV, v));
-            V::fma(acc, a.w[k], s);
+            val[k - 1][0] = x - k >= rc.xmin ? V::ldg(own - (int64_t)k * SV) : V::zero();
+            val[k - 1][1] = x + k <= rc.xmax ? V::ldg(own + (int64_t)k * SV) : V::zero();
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int4 r = nr[4 * (k - 1) + j];
+                val[k - 1][2 + j] = x >= r.y && x <= r.z ? V::ldg(in + (int64_t)(r.x + x) * SV + v) : V::zero();
+            }
         }
-        finish_point<R>(a, idx, x, y, z, v, c, acc);
+        double2 acc = V::scale(3.0 * a.w[0], c);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            double2 s = V::add(val[k][0], val[k][1]);
+#pragma unroll
+            for (int j = 2; j < 6; j++) s = V::add(s, val[k][j]);
+            V::fma(acc, a.w[k + 1], s);
+        }
+        const double2 b = a.base != nullptr ? ((const double2 *)a.base)[idx * SV + v] : V::zero();
+        finish_fp64(a, idx, x, y, z, v, c, acc, a.V[idx], b, nl);
     }
+}
+
+// The plain kernel, complex64: one thread per column of (point, vector),
+// marching along z over zs planes with its nine z values in registers; the 16
+// neighbours along x and y come through L1.  A warp owns 32 consecutive
+// (point, vector) values of the bounding-box row (x fastest after the
+// vector), a block eight such rows, so that a y neighbour read by one warp is
+// in L1 for the others.  All loads of a plane are independent, and where
+// every lane's neighbours exist they carry no range checks.  Bound by
+// instruction issue and L1 latency at 16 warps per SM.  The sums keep one
+// order: per distance k the six values x-, x+, y-, y+, z-, z+, then the
+// weight.  Used where a mesh gives the tiled kernels too few blocks; zs is
+// small there, so that all SMs have warps.  64^3 x 2 columns: 12.9 us, 48^3 x
+// 16 states: 32.6 us (28.7 and 48.1 us with a row lookup per neighbour and 25
+// loads a value).
+constexpr int kNaiveTY = 8, kNaiveMaxZ = 32;
+template <typename R>
+__global__ void __launch_bounds__(32 * kNaiveTY, 2) k_apply_naive(const ApplyArgs<R> a, int zs) {
+    static_assert(sizeof(R) == 4, "complex64");
+    using V = VT<R>;
+    using T = typename V::T;
+    constexpr int WY = kNaiveTY + 8;
+    // rows y0 - 4 .. y0 + 11 of planes z0 - 4 .. z0 + zs + 3: start - xmin, xmin, xmax
+    __shared__ SRow rows[(kNaiveMaxZ + 8) * WY];
+    // x range of each output row whose 16 in-plane neighbours all exist
+    __shared__ int2 inner[kNaiveMaxZ * kNaiveTY];
+    const int ny = a.ny, nz = a.nz, SV = a.SV;
+    const int y0 = blockIdx.y * kNaiveTY, z0 = blockIdx.z * zs;
+    const int z1 = min(z0 + zs, nz);
+    const int tid = threadIdx.y * 32 + threadIdx.x;
+    for (int i = tid; i < (z1 - z0 + 8) * WY; i += 32 * kNaiveTY) {
+        const Row r = load_row(a.rows, y0 - 4 + i % WY, z0 - 4 + i / WY, ny, nz);
+        rows[i] = SRow{r.start - r.xmin, (int16_t)r.xmin, (int16_t)r.xmax};
+    }
+    __syncthreads();
+    for (int i = tid; i < (z1 - z0) * kNaiveTY; i += 32 * kNaiveTY) {
+        const SRow *r = rows + (i / kNaiveTY + 4) * WY + 4 + i % kNaiveTY;
+        int lo = r[0].xmin + 4, hi = r[0].xmax - 4;
+#pragma unroll
+        for (int k = 1; k <= 4; k++) {
+            lo = max(lo, max((int)r[-k].xmin, (int)r[k].xmin));
+            hi = min(hi, min((int)r[-k].xmax, (int)r[k].xmax));
+        }
+        inner[i] = make_int2(lo, hi);
+    }
+    __syncthreads();
+    const int f = blockIdx.x * 32 + threadIdx.x;
+    const int x = f / SV, v = f - x * SV, y = y0 + threadIdx.y;
+    const bool lane_ok = x < a.nx && y < ny;
+    const T *__restrict__ in = (const T *)a.in + v;
+    const SRow *own = rows + 4 + threadIdx.y;   // own row of plane z: own[(z - z0 + 4) * WY]
+    auto value = [&](const SRow &r, int xx) -> T {
+        return xx >= r.xmin && xx <= r.xmax ? V::ldg(in + (int64_t)(r.start + xx) * SV) : V::zero();
+    };
+    auto entries = [&](const SRow &r) {
+        return lane_ok && x >= r.xmin && x <= r.xmax ? load_projectors<R>(a, (int64_t)r.start + x) : NlPoint{0, 0, 0};
+    };
+    T q[9];
+#pragma unroll
+    for (int j = 0; j < 9; j++) q[j] = lane_ok ? value(own[j * WY], x) : V::zero();
+    NlPoint nl = entries(own[4 * WY]);
+#pragma unroll 1
+    for (int z = z0; z < z1; z++) {
+        const SRow *rz = own + (z - z0 + 4) * WY;
+        const SRow rc = rz[0];
+        const bool ok = lane_ok && x >= rc.xmin && x <= rc.xmax;
+        T nxt = V::zero();
+        if (lane_ok && z + 1 < z1) nxt = value(rz[5 * WY], x);
+        // the next plane's projector entries, a plane ahead of their use
+        NlPoint nl1{0, 0, 0};
+        if (a.nl_ptr != nullptr) nl1 = entries(rz[WY]);
+        if (ok) {
+            const int64_t idx = (int64_t)rc.start + x;
+            const T *pc = in + idx * SV;
+            const R vloc = a.V[idx];
+            T bval = V::zero();
+            if (a.base != nullptr) bval = ((const T *)a.base)[idx * SV + v];
+            const int2 inr = inner[(z - z0) * kNaiveTY + threadIdx.y];
+            T val[4][4];
+            if (__all_sync(__activemask(), x >= inr.x && x <= inr.y)) {
+#pragma unroll
+                for (int k = 1; k <= 4; k++) {
+                    val[k - 1][0] = V::ldg(pc - (int64_t)(k * SV));
+                    val[k - 1][1] = V::ldg(pc + (int64_t)(k * SV));
+                    val[k - 1][2] = V::ldg(in + (int64_t)(rz[-k].start + x) * SV);
+                    val[k - 1][3] = V::ldg(in + (int64_t)(rz[k].start + x) * SV);
+                }
+            } else {
+#pragma unroll
+                for (int k = 1; k <= 4; k++) {
+                    val[k - 1][0] = value(rc, x - k);
+                    val[k - 1][1] = value(rc, x + k);
+                    val[k - 1][2] = value(rz[-k], x);
+                    val[k - 1][3] = value(rz[k], x);
+                }
+            }
+            T acc = V::scale((R)3 * a.w[0], q[4]);
+#pragma unroll
+            for (int k = 1; k <= 4; k++) {
+                T s = V::add(val[k - 1][0], val[k - 1][1]);
+                s = V::add(s, val[k - 1][2]);
+                s = V::add(s, val[k - 1][3]);
+                s = V::add(s, q[4 - k]);
+                s = V::add(s, q[4 + k]);
+                V::fma(acc, a.w[k], s);
+            }
+            finish_point<R>(a, idx, x, y, z, v, q[4], acc, vloc, bval, nl);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; j++) q[j] = q[j + 1];
+        q[8] = nxt;
+        nl = nl1;
+    }
+}
+
+// Planes per block: the number that gives the shortest schedule, rounds of
+// two blocks per SM times planes (plus two for the start of a block, which
+// reads the nine planes around its first one).
+inline int naive_zs(long long blocks_per_plane, int nz) {
+    int best = 1;
+    long long cost = INT64_MAX;
+    for (int zs = 1; zs <= kNaiveMaxZ && zs <= nz; zs++) {
+        const long long blocks = blocks_per_plane * ((nz + zs - 1) / zs);
+        const long long c = (blocks + 303) / 304 * (zs + 2);
+        if (c < cost) {
+            cost = c;
+            best = zs;
+        }
+    }
+    return best;
 }
 
 // One thread per (point, vector) with the antisymmetric-image boundary of a
@@ -667,7 +899,15 @@ static cudaError_t launch_staged_cv(const ApplyArgs<R> &a, const TileCfg &cfg, i
 template <typename R>
 cudaError_t launch_apply(const ApplyArgs<R> &a, const TileCfg &cfg, int ntiles, cudaStream_t st) {
     if (cfg.kernel == 1) {
-        k_apply_naive<R><<<a.ny * a.nz, 256, 0, st>>>(a);
+        if constexpr (sizeof(R) == 8) {
+            const long long per_row = ((long long)a.nx * a.SV + kRowNT - 1) / kRowNT;
+            k_apply_row64<R><<<dim3(a.ny * a.nz, (unsigned)(per_row < 65535 ? per_row : 65535)), kRowNT, 0, st>>>(a);
+        } else {
+            const long long gx = ((long long)a.nx * a.SV + 31) / 32;
+            if (gx > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+            const int gy = (a.ny + kNaiveTY - 1) / kNaiveTY, zs = naive_zs(gx * gy, a.nz);
+            k_apply_naive<R><<<dim3((unsigned)gx, gy, (a.nz + zs - 1) / zs), dim3(32, kNaiveTY), 0, st>>>(a, zs);
+        }
         return cudaGetLastError();
     }
     if (ntiles == 0) return cudaSuccess;
