@@ -163,6 +163,7 @@ struct rsg_mesh_s {
     // tile lists keyed by (TX, TY, zseg): device tiles and their count
     std::map<std::tuple<int, int, int>, std::pair<DevBuf, int>> tiles;
     std::map<std::tuple<int, int, int>, std::vector<Tile>> tiles_host;   // the same lists on the host
+    std::map<std::pair<int, int>, std::vector<int>> col_len;   // planes of every TX x TY column of tiles
 };
 
 struct rsg_ham_s {
@@ -175,6 +176,9 @@ struct rsg_ham_s {
     double proj_norm = 0.0;            // bound on the non-local operator: sum over atoms of sum |h_ij|
     TileCfg cfg;
     bool force_kernel = false;   // set when the caller chose the kernel explicitly
+    // complex64: the kernel and segment length chosen per (vectors per point,
+    // complex scaling, projectors) in the default configuration
+    std::map<std::tuple<int, bool, bool>, TileCfg> auto_cfg;
     int last_kernel = -1;        // stencil kernel of the last application
     int adj_keep = -1;           // adjoint: keep segment powers (1), recompute (0), by memory (-1)
     int adj_merge = -1;          // adjoint: costate and recompute sweeps share launches (1), not (0), auto (-1)
@@ -406,6 +410,132 @@ int tiles_for(rsg_ham H, const TileCfg &c, int SV, const Tile **tiles) {
     return n;
 }
 
+// ------------------------------------------- kernel choice, complex64 ----
+// Default configuration: kernel 7, 16 x 6 tiles, four producer warps,
+// 190-plane segments.
+TileCfg c64_config() {
+    TileCfg c;
+    c.kernel = 7;
+    c.wty = 6;
+    c.npw = 4;
+    c.threads = 192;
+    c.zseg = 190;
+    c.stages = 3;
+    return c;
+}
+bool default_c64(const TileCfg &c) {
+    const TileCfg d = c64_config();
+    return c.kernel == d.kernel && c.wty == d.wty && c.npw == d.npw && c.threads == d.threads && c.zseg == d.zseg &&
+           c.stages == d.stages && c.sync == d.sync;
+}
+
+// Planes of every TX x TY column of tiles that holds mesh points, longest
+// first.
+const std::vector<int> &column_lengths(rsg_mesh m, int TX, int TY) {
+    auto it = m->col_len.find({TX, TY});
+    if (it != m->col_len.end()) return it->second;
+    const int ntx = (m->nx + TX - 1) / TX, nty = (m->ny + TY - 1) / TY;
+    std::vector<int> zlo((size_t)ntx * nty, m->nz), zhi((size_t)ntx * nty, 0);
+    for (int z = 0; z < m->nz; z++)
+        for (int y = 0; y < m->ny; y++) {
+            const Row &r = m->rows[(size_t)z * m->ny + y];
+            if (r.xmin > r.xmax) continue;
+            for (int tx = r.xmin / TX; tx <= r.xmax / TX; tx++) {
+                const size_t k = (size_t)(y / TY) * ntx + tx;
+                zlo[k] = std::min(zlo[k], z);
+                zhi[k] = z + 1;
+            }
+        }
+    std::vector<int> len;
+    for (size_t k = 0; k < zlo.size(); k++)
+        if (zhi[k] > zlo[k]) len.push_back(zhi[k] - zlo[k]);
+    std::sort(len.rbegin(), len.rend());
+    return m->col_len[{TX, TY}] = len;
+}
+
+// Planes until the last of `slots` resident blocks is done: columns cut into
+// segments of zs planes (plus 8 planes of halo each), nch blocks per segment,
+// longest first to the first free slot; *blocks receives their number.
+double makespan(const std::vector<int> &col, int zs, int nch, int slots, int64_t *blocks) {
+    std::map<int, int64_t, std::greater<int>> by_len;   // planes -> blocks
+    int64_t n = 0, total = 0;
+    for (int L : col)
+        for (int z = 0; z < L; z += zs) {
+            const int len = std::min(zs, L - z) + 8;
+            by_len[len] += nch;
+            n += nch;
+            total += (int64_t)len * nch;
+        }
+    *blocks = n;
+    if (n == 0) return 0.0;
+    if (n > 16 * (int64_t)slots) return (double)total / slots + 0.5 * by_len.begin()->first;
+    std::vector<int64_t> heap((size_t)slots, 0);   // min-heap of finish times
+    int64_t last = 0;
+    for (const auto &b : by_len)
+        for (int64_t k = 0; k < b.second; k++) {
+            std::pop_heap(heap.begin(), heap.end(), std::greater<int64_t>());
+            heap.back() += b.first;
+            last = std::max(last, heap.back());
+            std::push_heap(heap.begin(), heap.end(), std::greater<int64_t>());
+        }
+    return (double)last;
+}
+
+// Stencil kernel and segment length of the default complex64 configuration.
+// The tiled kernels march whole columns, so a block takes about a microsecond
+// per plane whatever its chunk holds, and a mesh of few columns leaves SMs
+// idle unless the columns are cut, which costs eight halo planes a cut; the
+// plain kernel has no halo and no minimum, but costs 30 ps a vector.  The
+// rule takes the smallest of these times, fitted to 14 meshes from 24^3 to
+// the R = 14 sphere with 2 to 64 states (us): kernel 7, one block per SM,
+// 0.97 a plane; kernel 5, two blocks per SM, 1.2 a plane, 0.92 with at most
+// one block per SM; the plain kernel 5 + 30e-6 per vector (a fifth more with
+// projectors in its epilogue, where the tiled kernels launch a scatter, 6 us;
+// the plain complex-scaled kernel 10 + 40e-6).  Measured against the plain
+// kernel, which all of these ran before: R = 10 sphere, 14 values a point:
+// 64 us (115); 96^3 x 16: 78 (168); 48^3 x 16: 19 (27); R = 14 sphere x 8:
+// 107 (173); 64^3 x 2: the plain kernel, 12.5 (21).
+TileCfg choose_c64(rsg_ham H, int SV) {
+    const std::tuple<int, bool, bool> key(SV, H->has_scaling, H->pj.natoms > 0);
+    auto it = H->auto_cfg.find(key);
+    if (it != H->auto_cfg.end()) return it->second;
+    rsg_mesh m = H->m;
+    TileCfg best = H->cfg, c5 = H->cfg;
+    c5.kernel = 5;
+    c5.threads = 192;
+    c5.stages = 3;
+    c5.sync = 0;
+    int tx7, ty7, tx5, ty5;
+    block_shape(H->cfg, SV, &tx7, &ty7);
+    block_shape(c5, SV, &tx5, &ty5);
+    const std::vector<int> &col7 = column_lengths(m, tx7, ty7), &col5 = column_lengths(m, tx5, ty5);
+    const int nch7 = (SV + 7) / 8, nch5 = (SV + 1) / 2;
+    const bool nl = H->pj.natoms > 0;
+    int64_t n = 0;
+    makespan(col7, best.zseg, nch7, 152, &n);
+    if (SV % 8 != 0 || n < 4 * 152) {
+        const double vec = (double)m->P * SV, tiled = nl ? 8.0 : 2.0;
+        double cost = H->has_scaling ? 10.0 + 40e-6 * vec : (5.0 + 30e-6 * vec) * (nl ? 1.2 : 1.0);
+        best.kernel = 1;
+        for (int zs : {190, 150, 96, 64, 48, 32, 24, 16, 12, 8}) {
+            const double m7 = makespan(col7, zs, nch7, 152, &n);
+            if (tiled + 0.97 * m7 < cost) {
+                cost = tiled + 0.97 * m7;
+                best = H->cfg;
+                best.zseg = zs;
+            }
+            const double m5 = makespan(col5, zs, nch5, 304, &n);
+            const double t5 = tiled + (n <= 152 ? 0.92 : 1.2) * m5;
+            if (zs <= 150 && t5 < cost) {
+                cost = t5;
+                best = c5;
+                best.zseg = zs;
+            }
+        }
+    }
+    return H->auto_cfg[key] = best;
+}
+
 // ------------------------------------------------------------ checks ----
 rsg_status check_block(rsg_ham H, const void *p, int64_t S, int64_t ld, const char *what) {
     if (!p) return fail(RSG_ERR_ARG, "%s is NULL", what);
@@ -435,6 +565,9 @@ struct Epi {
     // (ar1, ai1); column 0 the call's eps and (ar, ai)
     bool twocol = false;
     double eps1 = 0, ar1 = 1, ai1 = 0;
+    // complex64: keep the kernel that applications of this shape have always
+    // run, whose sums fix every rounding (the solvers, which amplify it)
+    bool fixed_kernel = false;
 };
 
 // A potential is set: the real V, or the complex v_theta of complex scaling.
@@ -530,14 +663,17 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
     int ntiles = 0;
     a.tiles = nullptr;
     TileCfg cfg = H->cfg;
+    const int ldc_v = SV * (int)(16 / cbytes(H->dtype));
+    const bool chosen = H->dtype == RSG_C64 && !H->force_kernel && !ep.fixed_kernel && !ep.twocol &&
+                        m->bc == RSG_BC_ZERO && default_c64(H->cfg);
+    if (chosen) cfg = choose_c64(H, SV);
     // kernel 7 moves 16-value chunks of each point row: blocks whose rows are
     // narrow or end in a mostly empty chunk take the register-blocked kernel
     // in its default shape unless kernel 7 was chosen explicitly; complex
     // scaling runs on kernel 7 in its default shape only
-    if (cfg.kernel == 7) {
-        const int ldc = SV * (int)(16 / cbytes(H->dtype));
+    if (cfg.kernel == 7 && !chosen) {
         if ((H->has_scaling && (cfg.wty != 6 || cfg.npw != 4)) ||
-            (!H->force_kernel && ldc % 16 != 0 && ldc < 40)) {
+            (!H->force_kernel && ldc_v % 16 != 0 && ldc_v < 40)) {
             cfg.kernel = 5;
             cfg.threads = 192;
             cfg.zseg = 150;
@@ -553,7 +689,7 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
         int TX, TY;
         block_shape(cfg, SV, &TX, &TY);
         CKS(get_tiles(m, TX, TY, cfg.zseg, &a.tiles, &ntiles));
-        if (cfg.kernel != 1 && cfg.kernel != 2 && !H->force_kernel) {
+        if (cfg.kernel != 1 && cfg.kernel != 2 && !H->force_kernel && !chosen) {
             // the staged kernel runs one block per SM: small problems that
             // give fewer than two blocks per SM go to the one-thread-per-value
             // kernel instead
@@ -909,16 +1045,10 @@ rsg_status rsg_ham_create(rsg_mesh m, rsg_dtype dtype, rsg_ham *out) {
     // kernel (16 x 6 tiles, four producer warps, 190-plane segments: fastest
     // on the sphere workloads measured); narrow blocks and complex scaling
     // run the register-blocked kernel (apply_t)
-    if (dtype == RSG_C128) {
+    if (dtype == RSG_C128)
         H->cfg.kernel = 1;
-    } else {
-        H->cfg.kernel = 7;
-        H->cfg.wty = 6;
-        H->cfg.npw = 4;
-        H->cfg.threads = 192;
-        H->cfg.zseg = 190;
-        H->cfg.stages = 3;
-    }
+    else
+        H->cfg = c64_config();
     *out = H;
     return RSG_OK;
 }
@@ -1825,8 +1955,12 @@ rsg_status rsg_eigensolve(rsg_ham H, void *psi, int64_t S, int64_t ld, int64_t n
 
     std::vector<std::complex<double>> A((size_t)S * S), Q;
     std::vector<double> lam, res((size_t)S);
+    // Ritz vectors of close levels amplify a change of rounding: complex64
+    // results stay those of one kernel
+    Epi plain;
+    plain.fixed_kernel = true;
     auto rayleigh_ritz = [&]() -> rsg_status {
-        Epi ep;
+        Epi ep = plain;
         CKS(apply(H, psi, H->w0.p, SV, H->eps, H->dir, ep, st));
         if (H->dtype == RSG_C64)
             CK(launch_cross_gram<float>(psi, H->w0.p, P, (int)ld, (int)S, h3, H->red.as<double>(), nbg,
@@ -1886,14 +2020,14 @@ rsg_status rsg_eigensolve(rsg_ham H, void *psi, int64_t S, int64_t ld, int64_t n
         const double sigma1 = sigma, gamma = 2.0 / sigma1;
         void *X = psi, *Y = H->w0.p, *Z = H->w1.p;
         {
-            Epi ep;                      // Y = (sigma1 / e) (H - c) X
+            Epi ep = plain;              // Y = (sigma1 / e) (H - c) X
             ep.ar = sigma1 / e;
             ep.shift = c;
             CKS(apply(H, X, Y, SV, H->eps, H->dir, ep, st));
         }
         for (int k = 2; k <= degree; k++) {
             const double sigma2 = 1.0 / (gamma - sigma);
-            Epi ep;                      // Z = (2 sigma2 / e) (H - c) Y - sigma sigma2 X
+            Epi ep = plain;              // Z = (2 sigma2 / e) (H - c) Y - sigma sigma2 X
             ep.ar = 2.0 * sigma2 / e;
             ep.shift = c;
             ep.base = X;
@@ -1957,6 +2091,9 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
         ep.base = in;
         ep.br = -zr;
         ep.bi = -zi;
+        // in complex64 the iterates amplify a change of rounding by orders of
+        // magnitude: results stay those of one kernel
+        ep.fixed_kernel = true;
         return apply(H, in, out, SV, H->eps, H->dir, ep, st);
     };
     auto comb = [&](const void *u, const void *v, void *w, const double *a, const double *bb) -> rsg_status {
