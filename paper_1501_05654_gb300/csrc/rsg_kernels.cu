@@ -946,6 +946,16 @@ cudaError_t launch_apply(const ApplyArgs<R> &a, const TileCfg &cfg, int ntiles, 
 // (per vector slice blockIdx.y), and the last block of an atom sums the
 // atom's chunks in chunk order, scales by h^3 and applies h_a, exactly as
 // k_proj_reduce does, then resets the counter for the next launch.
+//
+// The chunk's point indices and projector values are staged first, so that a
+// lane's state loads (UNR in flight) depend on nothing but shared memory; the
+// lane sums of all projectors are left in shared memory and every (projector,
+// component, vector) is added up by its own thread, lanes in order.  Bound by
+// the latency of the gathered loads and of the FP64 additions.  One thread
+// per vector used to add the lanes of one projector at a time: one atom, one
+// vector a point 48 to 18 us; R = 18 sphere, 32 atoms x 4
+// projectors, 64 states 51 to 44 us; 192^3, 64 x 9, 128 states 0.59 to 0.46 ms.
+constexpr int kDotChunk = 512;   // entries of a chunk (the host cuts them)
 template <typename R, int NP>
 __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__restrict__ u, int SV,
                                                   const int32_t *__restrict__ q_pt,
@@ -960,54 +970,58 @@ __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__res
     using V = VT<R>;
     using T = typename V::T;
     constexpr int NCOMP = 2 * V::NC;
-    __shared__ double red[256 * NCOMP];
-    const int c = blockIdx.x;
-    const int v = blockIdx.y * blockDim.x + threadIdx.x;
-    const int q0 = chunk_q0[c], q1 = chunk_q1[c];
+    // projector values of the chunk, then the lane sums, then the atom's c
+    __shared__ __align__(16) unsigned char sm[NP * NCOMP * 256 * sizeof(R)];
+    __shared__ int qs[kDotChunk];
+    static_assert(kDotChunk * NP * sizeof(R) <= sizeof(sm) && 2 * NP * 32 * V::NC * sizeof(double) <= sizeof(sm), "");
+    R *qv = (R *)sm, *red = (R *)sm;
+    double *cbuf = (double *)sm;   // c[i][s] of the slice (re, im)
+    const int c = blockIdx.x, bx = blockDim.x, by = blockDim.y;
+    const int v = blockIdx.y * bx + threadIdx.x;
+    const int tid = threadIdx.y * bx + threadIdx.x, nth = bx * by;
+    const int q0 = chunk_q0[c], nq = chunk_q1[c] - q0;
+    for (int i = tid; i < nq; i += nth) qs[i] = q_pt[q0 + i];
+    for (int i = tid; i < nq * NP; i += nth) qv[i] = q_p[(int64_t)q0 * NP + i];
+    __syncthreads();
     T acc[NP];
 #pragma unroll
     for (int i = 0; i < NP; i++) acc[i] = V::zero();
     if (v < SV) {
-        // UNR entries per iteration: their point indices, then their values,
-        // are independent loads in flight together
-        constexpr int UNR = 4;
-        const int by = blockDim.y;
-        int q = q0 + threadIdx.y;
-        for (; q + (UNR - 1) * by < q1; q += UNR * by) {
-            int pt[UNR];
-#pragma unroll
-            for (int k = 0; k < UNR; k++) pt[k] = q_pt[q + k * by];
+        constexpr int UNR = NP > 4 ? 4 : 8;
+        int q = threadIdx.y;
+        for (; q + (UNR - 1) * by < nq; q += UNR * by) {
             T val[UNR];
 #pragma unroll
-            for (int k = 0; k < UNR; k++) val[k] = V::ldg(u + (int64_t)pt[k] * SV + v);
+            for (int k = 0; k < UNR; k++) val[k] = V::ldg(u + (int64_t)qs[q + k * by] * SV + v);
 #pragma unroll
             for (int k = 0; k < UNR; k++)
 #pragma unroll
-                for (int i = 0; i < NP; i++) V::fma(acc[i], q_p[(int64_t)(q + k * by) * NP + i], val[k]);
+                for (int i = 0; i < NP; i++) V::fma(acc[i], qv[(q + k * by) * NP + i], val[k]);
         }
-        for (; q < q1; q += by) {
-            const T val = V::ldg(u + (int64_t)q_pt[q] * SV + v);
+        // the rest, its loads in flight together too
+        T val[UNR];
 #pragma unroll
-            for (int i = 0; i < NP; i++) V::fma(acc[i], q_p[(int64_t)q * NP + i], val);
-        }
+        for (int k = 0; k < UNR; k++)
+            val[k] = q + k * by < nq ? V::ldg(u + (int64_t)qs[q + k * by] * SV + v) : V::zero();
+#pragma unroll
+        for (int k = 0; k < UNR; k++)
+            if (q + k * by < nq)
+#pragma unroll
+                for (int i = 0; i < NP; i++) V::fma(acc[i], qv[(q + k * by) * NP + i], val[k]);
     }
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    for (int i = 0; i < NP; i++) {
+    __syncthreads();   // the projector values have been read
 #pragma unroll
-        for (int j = 0; j < NCOMP; j++) red[tid * NCOMP + j] = (double)V::comp(acc[i], j);
-        __syncthreads();
-        if (threadIdx.y == 0 && v < SV) {
-            double s[NCOMP];
+    for (int i = 0; i < NP; i++)
 #pragma unroll
-            for (int j = 0; j < NCOMP; j++) s[j] = 0.0;
-            for (int l = 0; l < (int)blockDim.y; l++)
-#pragma unroll
-                for (int j = 0; j < NCOMP; j++) s[j] += red[(l * blockDim.x + threadIdx.x) * NCOMP + j];
-            double *dst = partial + (((int64_t)c * NP + i) * SV + v) * NCOMP;
-#pragma unroll
-            for (int j = 0; j < NCOMP; j++) dst[j] = s[j];
-        }
-        __syncthreads();
+        for (int j = 0; j < NCOMP; j++) red[(i * NCOMP + j) * 256 + tid] = V::comp(acc[i], j);
+    __syncthreads();
+    for (int t = tid; t < NP * NCOMP * bx; t += nth) {
+        const int ij = t / bx, x = t - ij * bx, vv = blockIdx.y * bx + x;
+        if (vv >= SV) continue;
+        double s = 0.0;
+#pragma unroll 8
+        for (int l = 0; l < by; l++) s += (double)red[ij * 256 + l * bx + x];
+        partial[(((int64_t)c * NP + ij / NCOMP) * SV + vv) * NCOMP + ij % NCOMP] = s;
     }
     if (counter == nullptr) return;
     // the last block of this atom and vector slice finishes its coefficients
@@ -1025,22 +1039,25 @@ __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__res
     if (!last) return;
     __threadfence();
     const int ldc = SV * V::NC;
-    const int s0 = blockIdx.y * blockDim.x * V::NC;                 // first complex column of the slice
-    const int ns = min((int)blockDim.x * V::NC, ldc - s0);          // complex columns in the slice
-    __shared__ double cbuf[2 * NP * 32 * V::NC];                    // c[i][s] of the slice (re, im)
-    for (int t = tid; t < NP * ns; t += blockDim.x * blockDim.y) {
-        const int i = t / ns, sc = s0 + (t - i * ns);
-        double sr = 0.0, si = 0.0;
-        for (int cc = atom_chunk0[at]; cc < atom_chunk0[at + 1]; cc++) {
-            const double *pp = partial + (((int64_t)cc * NP + i) * ldc + sc) * 2;
-            sr += __ldcg(pp);
-            si += __ldcg(pp + 1);
+    const int s0 = blockIdx.y * bx * V::NC;                 // first complex column of the slice
+    const int ns = min(bx * V::NC, ldc - s0);               // complex columns in the slice
+    const int c0 = atom_chunk0[at], c1 = atom_chunk0[at + 1];
+    for (int t = tid; t < NP * ns * 2; t += nth) {
+        const int i = t / (2 * ns), sc = t - i * 2 * ns;   // real or imaginary part of a column
+        const double *pp = partial + ((int64_t)i * ldc + s0) * 2 + sc;
+        double sum = 0.0;
+        for (int cc = c0; cc < c1; cc += 8) {   // eight loads in flight, added in order
+            double p[8];
+#pragma unroll
+            for (int k = 0; k < 8; k++) p[k] = cc + k < c1 ? __ldcg(pp + (int64_t)(cc + k) * NP * ldc * 2) : 0.0;
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                if (cc + k < c1) sum += p[k];
         }
-        cbuf[2 * t] = h3 * sr;
-        cbuf[2 * t + 1] = h3 * si;
+        cbuf[t] = h3 * sum;
     }
     __syncthreads();
-    for (int t = tid; t < NP * ns; t += blockDim.x * blockDim.y) {
+    for (int t = tid; t < NP * ns; t += nth) {
         const int i = t / ns, sl = t - i * ns;
         double dr = 0.0, di = 0.0;
         for (int j = 0; j < NP; j++) {
