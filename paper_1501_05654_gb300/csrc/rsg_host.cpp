@@ -177,7 +177,8 @@ struct rsg_ham_s {
     TileCfg cfg;
     bool force_kernel = false;   // set when the caller chose the kernel explicitly
     // complex64: the kernel and segment length chosen per (vectors per point,
-    // complex scaling, projectors) in the default configuration
+    // complex scaling, projectors) in the default configuration; complex128:
+    // the sums and planes per block of kernel 1, per vectors per point
     std::map<std::tuple<int, bool, bool>, TileCfg> auto_cfg;
     int last_kernel = -1;        // stencil kernel of the last application
     int adj_keep = -1;           // adjoint: keep segment powers (1), recompute (0), by memory (-1)
@@ -454,14 +455,14 @@ const std::vector<int> &column_lengths(rsg_mesh m, int TX, int TY) {
 }
 
 // Planes until the last of `slots` resident blocks is done: columns cut into
-// segments of zs planes (plus 8 planes of halo each), nch blocks per segment,
+// segments of zs planes (plus halo planes each), nch blocks per segment,
 // longest first to the first free slot; *blocks receives their number.
-double makespan(const std::vector<int> &col, int zs, int nch, int slots, int64_t *blocks) {
+double makespan(const std::vector<int> &col, int zs, int nch, int slots, int64_t *blocks, int halo = 8) {
     std::map<int, int64_t, std::greater<int>> by_len;   // planes -> blocks
     int64_t n = 0, total = 0;
     for (int L : col)
         for (int z = 0; z < L; z += zs) {
-            const int len = std::min(zs, L - z) + 8;
+            const int len = std::min(zs, L - z) + halo;
             by_len[len] += nch;
             n += nch;
             total += (int64_t)len * nch;
@@ -534,6 +535,36 @@ TileCfg choose_c64(rsg_ham H, int SV) {
         }
     }
     return H->auto_cfg[key] = best;
+}
+
+// complex128: planes per block of the integer-sum kernel, or 0 for FP64 sums,
+// by the smaller of two fitted times (us): FP64 sums 6 + 125e-6 per value; the
+// integer kernel 3 plus its schedule, a block (two per SM) taking 5 a plane
+// and 5 to start, 3.2 a plane with at most one block per SM.  24^3 x 1: 8.8
+// and 9.2 (FP64 sums); R = 5 sphere x 5: 51 and 49; 32^3 x 4: 21 and 17; 96^3
+// x 3: 325 and 179.
+int choose_c128(rsg_ham H, int SV) {
+    const std::tuple<int, bool, bool> key(SV, false, false);
+    auto it = H->auto_cfg.find(key);
+    if (it != H->auto_cfg.end()) return it->second.sum_zs;
+    int tx, ty;
+    sum64_shape(SV, &tx, &ty);
+    const std::vector<int> &col = column_lengths(H->m, tx, ty);
+    const int ns = sum64_states(SV), nch = (SV + ns - 1) / ns;
+    TileCfg best = H->cfg;
+    best.sum_zs = 0;
+    double cost = 6.0 + 125e-6 * (double)H->m->P * SV;
+    for (int zs : {32, 24, 16, 12, 8, 6, 4, 3, 2, 1}) {
+        int64_t n = 0;
+        const double mk = makespan(col, zs, nch, 304, &n, 1);
+        const double t = 3.0 + (n <= 152 ? 3.2 : 5.0) * mk;
+        if (t < cost) {
+            cost = t;
+            best.sum_zs = zs;
+        }
+    }
+    H->auto_cfg[key] = best;
+    return best.sum_zs;
 }
 
 // ------------------------------------------------------------ checks ----
@@ -685,6 +716,8 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
     if ((cfg.kernel == 2 || cfg.kernel == 3) && cfg.zseg > 120) cfg.zseg = 120;
     // two-column applications run on the one-thread-per-value kernel
     if (ep.twocol) cfg.kernel = 1;
+    if (H->dtype == RSG_C128 && cfg.kernel == 1 && m->bc == RSG_BC_ZERO && !H->has_scaling)
+        cfg.sum_zs = choose_c128(H, SV);
     if (cfg.kernel != 1) {
         int TX, TY;
         block_shape(cfg, SV, &TX, &TY);

@@ -39,6 +39,7 @@ struct TileCfg {
     int blocks_per_sm = 2;   // staged kernel, 256 threads: register budget for 2 or 3 blocks per SM
     int sync = 0;     // kernel 5, 192 threads: 0 block barrier per plane, 1/2 per-slot mbarriers
     int threads = 256;   // staged kernel: threads per block (256 with two blocks per SM, or 512)
+    int sum_zs = 0;      // kernel 1, complex128: planes per block of the integer-sum kernel (0: FP64 sums)
 };
 
 // Facts about an application that its FP64 epilogue uses (ApplyArgs::ef).
@@ -138,6 +139,11 @@ cudaError_t launch_apply_rowtma(const ApplyArgs<R> &a, const TileCfg &cfg, int n
 template <typename R>
 cudaError_t launch_apply(const ApplyArgs<R> &a, const TileCfg &cfg, int ntiles,
                          cudaStream_t st);
+// complex128 stencil with integer neighbour sums (rsg_sum64.cu): zs planes per
+// block (1..32), tile and states per block for SV vectors per point.
+cudaError_t launch_apply_sum64(const ApplyArgs<double> &a, int zs, cudaStream_t st);
+void sum64_shape(int SV, int *TX, int *TY);
+int sum64_states(int SV);
 // Complex-scaled operator -1/2 e^{-2i theta} lap + v_theta (+ the real
 // constant a.f0): vt holds the interleaved complex v_theta of every point;
 // a.nl_ptr and the field terms are ignored (rsg_scaled.cu).
