@@ -2113,12 +2113,10 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
     CK(H->red.ensure((size_t)nbn * S * 2 * sizeof(double)));
     CK(H->cg.ensure((size_t)S * 10 * sizeof(double)));
     double *cgb = H->cg.as<double>();
-    double *d_dot = cgb, *d_nrm = cgb + 2 * S, *d_a = cgb + 3 * S, *d_b = cgb + 5 * S, *d_one = cgb + 7 * S;
+    double *d_dot = cgb, *d_a = cgb + 2 * S, *d_b = cgb + 4 * S, *d_nrm = cgb + 6 * S;   // complex ones 16-byte aligned
     void *r = H->w0.p, *p = H->w1.p, *q = H->w2.p;
     const bool c64 = H->dtype == RSG_C64;
-    std::vector<double> one((size_t)2 * S, 0.0), coef((size_t)4 * S);
-    for (int64_t s = 0; s < S; s++) one[(size_t)2 * s] = 1.0;
-    CK(cudaMemcpyAsync(d_one, one.data(), (size_t)2 * S * sizeof(double), cudaMemcpyHostToDevice, st));
+    std::vector<double> coef((size_t)4 * S);
     auto Ax = [&](const void *in, void *out) -> rsg_status {     // out = (H - z) in
         Epi ep;
         ep.base = in;
@@ -2129,9 +2127,9 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
         ep.fixed_kernel = true;
         return apply(H, in, out, SV, H->eps, H->dir, ep, st);
     };
-    auto comb = [&](const void *u, const void *v, void *w, const double *a, const double *bb) -> rsg_status {
-        if (c64) CK(launch_comb<float>(u, v, w, P, (int)ld, (int)S, a, bb, st));
-        else CK(launch_comb<double>(u, v, w, P, (int)ld, (int)S, a, bb, st));
+    auto comb = [&](const void *u, const void *v, void *w, const double *bb) -> rsg_status {   // w = u + bb v
+        if (c64) CK(launch_comb<float>(u, v, w, P, (int)ld, (int)S, bb, st));
+        else CK(launch_comb<double>(u, v, w, P, (int)ld, (int)S, bb, st));
         return RSG_OK;
     };
     std::vector<double> dot((size_t)2 * S), nrm((size_t)S), bn((size_t)S);
@@ -2162,7 +2160,7 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
     CKS(Ax(x, q));
     for (int64_t s = 0; s < S; s++) neg[(size_t)s] = -1.0;
     CKS(upload(neg, d_a));
-    CKS(comb(b, q, r, d_one, d_a));
+    CKS(comb(b, q, r, d_a));
     CK(cudaMemcpyAsync(p, r, bytes, cudaMemcpyDeviceToDevice, st));
     CKS(norms(b, bn));
     CKS(bilinear(r, r));
@@ -2194,9 +2192,9 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
             neg[(size_t)s] = -alpha[(size_t)s];
         }
         CKS(upload(alpha, d_a));
-        CKS(comb(x, p, x, d_one, d_a));          // x += alpha p
+        CKS(comb(x, p, x, d_a));          // x += alpha p
         CKS(upload(neg, d_b));
-        CKS(comb(r, q, r, d_one, d_b));          // r -= alpha q
+        CKS(comb(r, q, r, d_b));          // r -= alpha q
         CKS(bilinear(r, r));
         CKS(norms(r, nrm));
         for (int64_t s = 0; s < S; s++) {
@@ -2205,14 +2203,14 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
             rho[(size_t)s] = rn;
         }
         CKS(upload(beta, d_b));
-        CKS(comb(r, p, p, d_one, d_b));          // p = r + beta p
+        CKS(comb(r, p, p, d_b));          // p = r + beta p
         it++;
     }
     // true residual |b - (H - z) x| / |b|
     CKS(Ax(x, q));
     for (int64_t s = 0; s < S; s++) neg[(size_t)s] = -1.0;
     CKS(upload(neg, d_a));
-    CKS(comb(b, q, r, d_one, d_a));
+    CKS(comb(b, q, r, d_a));
     CKS(norms(r, nrm));
     if (resid_out)
         for (int64_t s = 0; s < S; s++)

@@ -188,10 +188,10 @@ cudaError_t launch_bilinear(const void *x, const void *y, int64_t P, int ld, int
 // psi[p, s] *= M[p] (M: P values of the compute type), the first S states.
 template <typename R>
 cudaError_t launch_mask(void *psi, int64_t P, int ld, int S, const void *M, cudaStream_t st);
-// z = a x + b y per state, complex a[s], b[s] (device, interleaved doubles); z may alias x or y.
+// z = x + b y per state, complex b[s] (device, interleaved doubles, 16-byte aligned); z may alias x or y.
 template <typename R>
-cudaError_t launch_comb(const void *x, const void *y, void *z, int64_t P, int ld, int S, const double *a,
-                        const double *b, cudaStream_t st);
+cudaError_t launch_comb(const void *x, const void *y, void *z, int64_t P, int ld, int S, const double *b,
+                        cudaStream_t st);
 // out[s] = h3 sum_p |hx[p,s] - lam[s] x[p,s]|^2 (FP64; partial nblk * S doubles).
 template <typename R>
 cudaError_t launch_resid(const void *x, const void *hx, int64_t P, int ld, int S, const double *lam, double h3,

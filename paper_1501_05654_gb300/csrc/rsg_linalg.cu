@@ -98,68 +98,132 @@ __global__ void __launch_bounds__(256) k_resid(const R *__restrict__ x, const R 
     if (threadIdx.x == 0) partial[(int64_t)blockIdx.x * S + s] = red[0];
 }
 
+// FP32 <-> FP64 in integer arithmetic.  A conversion instruction takes two
+// slots of the FP64 pipe (two a clock per SM), which bounds the complex64
+// vector updates below; exponents that need denormal or special handling take
+// the instruction.  R = 14 sphere x 8 states: update 293 to 91 us (with the
+// unit scale of x dropped and 16-byte accesses), bilinear form 251 to 139 us.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return (u & 0x7fffffffu) == 0u ? __hiloint2double((int)u, 0) : (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double d) { return d; }
+// round to nearest even
+__device__ __forceinline__ float narrow(double d, float) {
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned e = hi & 0x7ff00000u;
+    // FP32 exponents 1 .. 253: normal, and a carry stays finite
+    if (e < 0x38100000u || e > 0x47d00000u) return (hi & 0x7fffffffu) == 0u && lo == 0u ? __uint_as_float(hi) : (float)d;
+    const unsigned m = ((hi & 0x7fffffffu) - 0x38000000u) << 3 | lo >> 29;   // truncated
+    const unsigned rest = lo & 0x1fffffffu;
+    return __uint_as_float((hi & 0x80000000u) | (m + (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u)))));
+}
+__device__ __forceinline__ double narrow(double d, double) { return d; }
+
 // partial[blk][s] (complex double) = sum over the block's points of
-// x[p,s] y[p,s] (the bilinear form of complex symmetric systems, no conjugate)
-template <typename R>
+// x[p,s] y[p,s] (the bilinear form of complex symmetric systems, no
+// conjugate).  A thread takes NS neighbouring states of every 256th point,
+// which a 16-byte load of complex64 brings together.
+template <typename R, int NS>
 __global__ void __launch_bounds__(256) k_bilinear(const R *__restrict__ x, const R *__restrict__ y, int64_t P,
                                                   int ld, int S, double *__restrict__ partial, int nblk) {
-    __shared__ double red[2][256];
-    const int s = blockIdx.y;
+    __shared__ double red[2 * NS][256];
+    const int s0 = blockIdx.y * NS;
     const int64_t per = (P + nblk - 1) / nblk;
     const int64_t p0 = blockIdx.x * per, p1 = p0 + per < P ? p0 + per : P;
-    double ar = 0.0, ai = 0.0;
-    for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        double xr, xi, yr, yi;
-        ld_c(x + (p * ld + s) * 2, xr, xi);
-        ld_c(y + (p * ld + s) * 2, yr, yi);
-        ar += xr * yr - xi * yi;
-        ai += xr * yi + xi * yr;
+    double ar[NS], ai[NS];
+#pragma unroll
+    for (int k = 0; k < NS; k++) ar[k] = ai[k] = 0.0;
+#pragma unroll 4
+    for (int64_t p = p0 + threadIdx.x; p < p1; p += 256) {
+        R xv[2 * NS], yv[2 * NS];
+        const R *xp = x + (p * ld + s0) * 2, *yp = y + (p * ld + s0) * 2;
+        if constexpr (NS == 2 && sizeof(R) == 4) {
+            const float4 a = *(const float4 *)xp, b = *(const float4 *)yp;
+            xv[0] = a.x, xv[1] = a.y, xv[2] = a.z, xv[3] = a.w;
+            yv[0] = b.x, yv[1] = b.y, yv[2] = b.z, yv[3] = b.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 2 * NS; k++) xv[k] = xp[k], yv[k] = yp[k];
+        }
+#pragma unroll
+        for (int k = 0; k < NS; k++) {
+            const double xr = widen(xv[2 * k]), xi = widen(xv[2 * k + 1]), yr = widen(yv[2 * k]),
+                         yi = widen(yv[2 * k + 1]);
+            ar[k] += xr * yr - xi * yi;
+            ai[k] += xr * yi + xi * yr;
+        }
     }
-    red[0][threadIdx.x] = ar;
-    red[1][threadIdx.x] = ai;
+#pragma unroll
+    for (int k = 0; k < NS; k++) {
+        red[2 * k][threadIdx.x] = ar[k];
+        red[2 * k + 1][threadIdx.x] = ai[k];
+    }
     __syncthreads();
     for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            red[0][threadIdx.x] += red[0][threadIdx.x + w];
-            red[1][threadIdx.x] += red[1][threadIdx.x + w];
-        }
+        if (threadIdx.x < w)
+#pragma unroll
+            for (int k = 0; k < 2 * NS; k++) red[k][threadIdx.x] += red[k][threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        partial[((int64_t)blockIdx.x * S + s) * 2] = red[0][0];
-        partial[((int64_t)blockIdx.x * S + s) * 2 + 1] = red[1][0];
-    }
+    if (threadIdx.x < 2 * NS && s0 + (int)threadIdx.x / 2 < S)
+        partial[((int64_t)blockIdx.x * S + s0) * 2 + threadIdx.x] = red[threadIdx.x][0];
 }
 
 template <typename R>
 cudaError_t launch_bilinear(const void *x, const void *y, int64_t P, int ld, int S, double h3, double *partial,
                             int nblk, double *out, cudaStream_t st) {
-    k_bilinear<R><<<dim3(nblk, S), 256, 0, st>>>((const R *)x, (const R *)y, P, ld, S, partial, nblk);
+    constexpr int NS = sizeof(R) == 4 ? 2 : 1;   // complex64 rows are whole 16-byte vectors
+    k_bilinear<R, NS><<<dim3(nblk, (S + NS - 1) / NS), 256, 0, st>>>((const R *)x, (const R *)y, P, ld, S, partial, nblk);
     return launch_sum_blocks(partial, nblk, 2 * (int64_t)S, h3, out, st);
 }
 
-// z[p,s] = a[s] x[p,s] + b[s] y[p,s] with complex per-state a, b (device,
-// interleaved doubles); z may alias x or y (each element is read before it
-// is written, by the same thread)
+// z[p,s] = x[p,s] + b[s] y[p,s] with complex per-state b (device, interleaved
+// doubles), in FP64 and rounded once; z may alias x or y (each element is
+// read before it is written, by the same thread).
 template <typename R>
 __global__ void __launch_bounds__(256) k_comb(const R *x, const R *y, R *z, int64_t P, int ld, int S,
-                                              const double *__restrict__ a, const double *__restrict__ b) {
+                                              const double *__restrict__ b) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= P * S) return;
-    const int64_t p = i / S;
-    const int s = (int)(i - p * S);
-    const int64_t o = (p * ld + s) * 2;
-    const double xr = (double)x[o], xi = (double)x[o + 1], yr = (double)y[o], yi = (double)y[o + 1];
-    const double ar = a[2 * s], ai = a[2 * s + 1], br = b[2 * s], bi = b[2 * s + 1];
-    z[o] = (R)(ar * xr - ai * xi + br * yr - bi * yi);
-    z[o + 1] = (R)(ar * xi + ai * xr + br * yi + bi * yr);
+    if constexpr (sizeof(R) == 4) {
+        // two states per thread
+        const int nv = (S + 1) / 2;
+        if (i >= P * nv) return;
+        const int64_t p = i / nv;
+        const int s = 2 * (int)(i - p * nv);
+        const int64_t o = (p * ld + s) * 2;
+        const float4 xv = *(const float4 *)(x + o), yv = *(const float4 *)(y + o);
+        const double2 b0 = *(const double2 *)(b + 2 * s);
+        const double y0r = widen(yv.x), y0i = widen(yv.y);
+        float4 r;
+        r.x = narrow(fma(-b0.y, y0i, fma(b0.x, y0r, widen(xv.x))), 0.f);
+        r.y = narrow(fma(b0.y, y0r, fma(b0.x, y0i, widen(xv.y))), 0.f);
+        if (s + 1 < S) {
+            const double2 b1 = *(const double2 *)(b + 2 * s + 2);
+            const double y1r = widen(yv.z), y1i = widen(yv.w);
+            r.z = narrow(fma(-b1.y, y1i, fma(b1.x, y1r, widen(xv.z))), 0.f);
+            r.w = narrow(fma(b1.y, y1r, fma(b1.x, y1i, widen(xv.w))), 0.f);
+            *(float4 *)(z + o) = r;
+        } else {
+            *(float2 *)(z + o) = make_float2(r.x, r.y);
+        }
+    } else {
+        if (i >= P * S) return;
+        const int64_t p = i / S;
+        const int s = (int)(i - p * S);
+        const int64_t o = (p * ld + s) * 2;
+        const double2 xv = *(const double2 *)(x + o), yv = *(const double2 *)(y + o);
+        const double br = b[2 * s], bi = b[2 * s + 1];
+        *(double2 *)(z + o) = make_double2(fma(-bi, yv.y, fma(br, yv.x, xv.x)), fma(bi, yv.x, fma(br, yv.y, xv.y)));
+    }
 }
 
 template <typename R>
-cudaError_t launch_comb(const void *x, const void *y, void *z, int64_t P, int ld, int S, const double *a,
-                        const double *b, cudaStream_t st) {
-    const int64_t n = P * S;
-    k_comb<R><<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const R *)x, (const R *)y, (R *)z, P, ld, S, a, b);
+cudaError_t launch_comb(const void *x, const void *y, void *z, int64_t P, int ld, int S, const double *b,
+                        cudaStream_t st) {
+    const int64_t n = P * (sizeof(R) == 4 ? (S + 1) / 2 : S);
+    k_comb<R><<<(unsigned)((n + 255) / 256), 256, 0, st>>>((const R *)x, (const R *)y, (R *)z, P, ld, S, b);
     return cudaGetLastError();
 }
 
@@ -552,7 +616,7 @@ cudaError_t launch_grad_accum(const double *M, double tau, double *grad_k, cudaS
     template cudaError_t launch_bilinear<R>(const void *, const void *, int64_t, int, int, double,   \
                                             double *, int, double *, cudaStream_t);                  \
     template cudaError_t launch_comb<R>(const void *, const void *, void *, int64_t, int, int,       \
-                                        const double *, const double *, cudaStream_t);               \
+                                        const double *, cudaStream_t);                               \
     template cudaError_t launch_mask<R>(void *, int64_t, int, int, const void *, cudaStream_t);      \
     template cudaError_t launch_tri_apply<R>(void *, int64_t, int, int, const double *,              \
                                              cudaStream_t);                                          \
