@@ -454,15 +454,15 @@ const std::vector<int> &column_lengths(rsg_mesh m, int TX, int TY) {
     return m->col_len[{TX, TY}] = len;
 }
 
-// Planes until the last of `slots` resident blocks is done: columns cut into
-// segments of zs planes (plus halo planes each), nch blocks per segment,
+// Time until the last of `slots` resident blocks is done: columns cut into
+// segments of zs planes, nch blocks per segment that take mul * planes + add,
 // longest first to the first free slot; *blocks receives their number.
-double makespan(const std::vector<int> &col, int zs, int nch, int slots, int64_t *blocks, int halo = 8) {
-    std::map<int, int64_t, std::greater<int>> by_len;   // planes -> blocks
+double makespan(const std::vector<int> &col, int zs, int nch, int slots, int64_t *blocks, int mul = 1, int add = 8) {
+    std::map<int, int64_t, std::greater<int>> by_len;   // time -> blocks
     int64_t n = 0, total = 0;
     for (int L : col)
         for (int z = 0; z < L; z += zs) {
-            const int len = std::min(zs, L - z) + halo;
+            const int len = mul * std::min(zs, L - z) + add;
             by_len[len] += nch;
             n += nch;
             total += (int64_t)len * nch;
@@ -539,10 +539,11 @@ TileCfg choose_c64(rsg_ham H, int SV) {
 
 // complex128: planes per block of the integer-sum kernel, or 0 for FP64 sums,
 // by the smaller of two fitted times (us): FP64 sums 6 + 125e-6 per value; the
-// integer kernel 3 plus its schedule, a block (two per SM) taking 5 a plane
-// and 5 to start, 3.2 a plane with at most one block per SM.  24^3 x 1: 8.8
-// and 9.2 (FP64 sums); R = 5 sphere x 5: 51 and 49; 32^3 x 4: 21 and 17; 96^3
-// x 3: 325 and 179.
+// integer kernel 3 plus its schedule over the SMs at 2.55 a plane (two blocks
+// share an SM's issue slots; a block starts in a fifth of a plane), at least
+// 3.2 a plane for a block by itself.  24^3 x 1: 8.8 and 9.2 us (FP64 sums taken);
+// R = 5 sphere x 5: 51 and 49; 32^3 x 4: 21 and 17; 61^3 x 8: 234 and 131 (8
+// planes a block; 148 with 32); 96^3 x 3: 325 and 179.
 int choose_c128(rsg_ham H, int SV) {
     const std::tuple<int, bool, bool> key(SV, false, false);
     auto it = H->auto_cfg.find(key);
@@ -556,8 +557,8 @@ int choose_c128(rsg_ham H, int SV) {
     double cost = 6.0 + 125e-6 * (double)H->m->P * SV;
     for (int zs : {32, 24, 16, 12, 8, 6, 4, 3, 2, 1}) {
         int64_t n = 0;
-        const double mk = makespan(col, zs, nch, 304, &n, 1);
-        const double t = 3.0 + (n <= 152 ? 3.2 : 5.0) * mk;
+        const double mk = makespan(col, zs, nch, 152, &n, 5, 1);
+        const double t = 3.0 + std::max(2.55 / 5 * mk, 3.2 * (col.empty() ? 0 : std::min(zs, col[0])));
         if (t < cost) {
             cost = t;
             best.sum_zs = zs;

@@ -8,6 +8,8 @@
 // complex64 update are in rsg_qr.cu).  The adjoint inner products of the
 // control gradient (Sec. "Quantum optimal control", Eq. (qoctgradient)) are
 // FP64 reductions as well.
+#include <algorithm>
+
 #include "rsg_internal.h"
 #include "rsg_vec.cuh"
 
@@ -23,52 +25,89 @@ __device__ __forceinline__ void ld_c(const R *p, double &re, double &im) {
 
 }  // namespace
 
-// psi[p, s] <- sum_t psi[p, t] Q[t][s] (Q: S x S complex double, the Ritz
-// rotation), in place: each block stages its full rows in shared memory.
-template <typename R>
-__global__ void __launch_bounds__(256) k_rotate(R *psi, int64_t P, int ld, int S, const double *__restrict__ Q,
-                                                int pt) {
-    extern __shared__ double rowbuf[];   // pt * S complex double
+// psi[p, s] <- sum_t psi[p, t] M[t][s] in place, FP64 sums: the Ritz rotation
+// (M = Q) or, TRI, the Cholesky-QR update (M[t][s] = conj(W[s][t]), t <= s).
+// A block stages the rows of PT points and chunks of M in shared memory; a
+// thread forms four neighbouring states of a point, so that 16 FP64 FMAs
+// share five 16-byte reads.  Bound by the FP64 pipe (two FMAs a clock per SM).
+constexpr int kRowsNT = 256, kRowsChunk = 2048;   // threads, complex values of M per chunk
+template <typename R, bool TRI>
+__global__ void __launch_bounds__(kRowsNT) k_rows(R *psi, int64_t P, int ld, int S, const double2 *__restrict__ M,
+                                                  int pt, int nt) {
+    extern __shared__ double2 rsm[];
+    double2 *rows = rsm, *mc = rsm + (size_t)pt * S;   // [pt][S], [nt][S]
+    const int tid = threadIdx.x, ng = (S + 3) / 4;
     const int64_t p0 = (int64_t)blockIdx.x * pt;
-    const int n = pt * S;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int q = e / S, t = e % S;
-        const int64_t p = p0 + q;
-        double re = 0.0, im = 0.0;
-        if (p < P) ld_c(psi + (p * ld + t) * 2, re, im);
-        rowbuf[e * 2] = re;
-        rowbuf[e * 2 + 1] = im;
+    for (int e = tid; e < pt * S; e += kRowsNT) {
+        const int q = e / S;
+        double2 v = make_double2(0.0, 0.0);
+        if (p0 + q < P) ld_c(psi + ((p0 + q) * ld + (e - q * S)) * 2, v.x, v.y);
+        rows[e] = v;
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int q = e / S, s = e % S;
-        const int64_t p = p0 + q;
-        if (p >= P) continue;
-        double re = 0.0, im = 0.0;
-        const double *row = rowbuf + (int64_t)q * S * 2;
-        for (int t = 0; t < S; t++) {
-            const double qr = Q[((int64_t)t * S + s) * 2], qi = Q[((int64_t)t * S + s) * 2 + 1];
-            re += row[2 * t] * qr - row[2 * t + 1] * qi;
-            im += row[2 * t] * qi + row[2 * t + 1] * qr;
+    // items (point, group of four states): pt * ng of them, kRowsNT at a time
+    for (int i0 = 0; i0 < pt * ng; i0 += kRowsNT) {
+        const int i = i0 + tid, q = i / ng, s0 = 4 * (i - q * ng);
+        const bool on = i < pt * ng && p0 + q < P;
+        double re[4] = {0.0, 0.0, 0.0, 0.0}, im[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int t0 = 0; t0 < S; t0 += nt) {
+            const int t1 = min(S, t0 + nt);
+            if (nt < S || i0 == 0) {   // a chunk that holds all of M is staged once
+                __syncthreads();
+                for (int e = tid; e < (t1 - t0) * S; e += kRowsNT) {
+                    const int t = t0 + e / S, s = e % S;
+                    double2 m;
+                    if (TRI) {
+                        m = t <= s ? M[(int64_t)s * S + t] : make_double2(0.0, 0.0);
+                        m.y = -m.y;
+                    } else {
+                        m = M[(int64_t)t * S + s];
+                    }
+                    mc[e] = m;
+                }
+                __syncthreads();
+            }
+            if (!on) continue;
+            const int te = TRI ? min(t1, s0 + 4) : t1;
+            const double2 *row = rows + (size_t)q * S;
+#pragma unroll 2
+            for (int t = t0; t < te; t++) {
+                const double2 a = row[t], *m = mc + (size_t)(t - t0) * S + s0;
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    const double2 w = s0 + k < S ? m[k] : make_double2(0.0, 0.0);
+                    re[k] = fma(a.x, w.x, fma(-a.y, w.y, re[k]));
+                    im[k] = fma(a.x, w.y, fma(a.y, w.x, im[k]));
+                }
+            }
         }
-        psi[(p * ld + s) * 2] = (R)re;
-        psi[(p * ld + s) * 2 + 1] = (R)im;
+        if (on)
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (s0 + k < S) {
+                    R *d = psi + ((p0 + q) * ld + s0 + k) * 2;
+                    d[0] = (R)re[k];
+                    d[1] = (R)im[k];
+                }
     }
+}
+
+template <typename R, bool TRI>
+cudaError_t rows_launch(void *psi, int64_t P, int ld, int S, const double *M, cudaStream_t st) {
+    // one item per thread, fewer points where the rows would not fit
+    const int ng = (S + 3) / 4, pt = std::max(1, kRowsNT / ng), nt = std::min(S, std::max(1, kRowsChunk / S));
+    const size_t smem = ((size_t)pt * S + (size_t)nt * S) * sizeof(double2);
+    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_rows<R, TRI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_rows<R, TRI><<<(unsigned)((P + pt - 1) / pt), kRowsNT, smem, st>>>((R *)psi, P, ld, S, (const double2 *)M, pt, nt);
+    return cudaGetLastError();
 }
 
 template <typename R>
 cudaError_t launch_rotate(void *psi, int64_t P, int ld, int S, const double *Q, cudaStream_t st) {
-    int pt = 4096 / S;
-    if (pt < 1) pt = 1;
-    if (pt > 64) pt = 64;
-    const size_t smem = (size_t)pt * S * 2 * sizeof(double);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_rotate<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    const int64_t nb = (P + pt - 1) / pt;
-    k_rotate<R><<<(unsigned)nb, 256, smem, st>>>((R *)psi, P, ld, S, Q, pt);
-    return cudaGetLastError();
+    return rows_launch<R, false>(psi, P, ld, S, Q, st);
 }
 
 // partial[blk][s] = sum over the block's points of |hx[p,s] - lam[s] x[p,s]|^2
@@ -254,53 +293,9 @@ cudaError_t launch_resid(const void *x, const void *hx, int64_t P, int ld, int S
     return launch_sum_blocks(partial, nblk, S, h3, out, st);
 }
 
-// psi[p, s] <- sum_{t <= s} psi[p, t] conj(W[s][t]); each block stages its
-// full rows in shared memory first, so the update is in place.
-template <typename R>
-__global__ void __launch_bounds__(256) k_tri_apply(R *psi, int64_t P, int ld, int S,
-                                                   const double *__restrict__ W, int pt) {
-    extern __shared__ double rowbuf[];   // pt * S complex double
-    const int64_t p0 = (int64_t)blockIdx.x * pt;
-    const int n = pt * S;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int q = e / S, t = e % S;
-        const int64_t p = p0 + q;
-        double re = 0.0, im = 0.0;
-        if (p < P) ld_c(psi + (p * ld + t) * 2, re, im);
-        rowbuf[e * 2] = re;
-        rowbuf[e * 2 + 1] = im;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int q = e / S, s = e % S;
-        const int64_t p = p0 + q;
-        if (p >= P) continue;
-        double re = 0.0, im = 0.0;
-        const double *row = rowbuf + (int64_t)q * S * 2;
-        for (int t = 0; t <= s; t++) {
-            const double wr = W[((int64_t)s * S + t) * 2], wi = -W[((int64_t)s * S + t) * 2 + 1];
-            re += row[2 * t] * wr - row[2 * t + 1] * wi;
-            im += row[2 * t] * wi + row[2 * t + 1] * wr;
-        }
-        psi[(p * ld + s) * 2] = (R)re;
-        psi[(p * ld + s) * 2 + 1] = (R)im;
-    }
-}
-
 template <typename R>
 cudaError_t launch_tri_apply(void *psi, int64_t P, int ld, int S, const double *W, cudaStream_t st) {
-    int pt = 4096 / S;
-    if (pt < 1) pt = 1;
-    if (pt > 64) pt = 64;
-    const size_t smem = (size_t)pt * S * 2 * sizeof(double);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_tri_apply<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    const int64_t nb = (P + pt - 1) / pt;
-    k_tri_apply<R><<<(unsigned)nb, 256, smem, st>>>((R *)psi, P, ld, S, W, pt);
-    return cudaGetLastError();
+    return rows_launch<R, true>(psi, P, ld, S, W, st);
 }
 
 // partial[blk][s] = sum over the block's points of |psi[p,s]|^2

@@ -360,6 +360,7 @@ __global__ void __launch_bounds__(256) k_gram64(const R *__restrict__ psi, const
     const int s0 = ti * kGD, t0 = tj * kGD;
     const int tid = threadIdx.x, g = tid / 16, r = tid % 16;
     const int sr = r / 4, tc = r % 4;   // rows sr, sr + 4; columns tc, tc + 4
+    const bool diag = herm && ti == tj;   // rows sr + 4, column tc: below the diagonal, not formed
     const int64_t per = (P + nblk - 1) / nblk;
     const int64_t p0 = blockIdx.z * per;
     const int64_t p1 = p0 + per < P ? p0 + per : P;
@@ -404,6 +405,7 @@ __global__ void __launch_bounds__(256) k_gram64(const R *__restrict__ psi, const
             for (int i = 0; i < 2; i++)
 #pragma unroll
                 for (int j = 0; j < 2; j++) {
+                    if (i == 1 && j == 0 && diag) continue;
                     acc[i][j].x = fma(x[i].x, y[j].x, fma(x[i].y, y[j].y, acc[i][j].x));
                     acc[i][j].y = fma(x[i].x, y[j].y, fma(-x[i].y, y[j].x, acc[i][j].y));
                 }
