@@ -23,7 +23,8 @@ SOURCES = [("rsg_kernels.cu", ["-DRSG_ONLY_FLOAT"]), ("rsg_kernels.cu", ["-DRSG_
            ("rsg_kernels.cu", ["-DRSG_ONLY_DOUBLE"]),
            ("rsg_quad.cu", []), ("rsg_wide.cu", []), ("rsg_bstep.cu", []), ("rsg_scaled.cu", []), ("rsg_selftest.cu", []), ("rsg_linalg.cu", []),
            ("rsg_qr.cu", []), ("rsg_sum64.cu", []), ("rsg_noalloc.cu", []), ("rsg_host.cpp", [])]
-HEADERS = ["rsg_internal.h", "rsg_vec.cuh", "rsg_async.cuh", "rsg_batch.cuh", "rsg_point.cuh"]
+HEADERS = ["rsg_internal.h", "rsg_vec.cuh", "rsg_async.cuh", "rsg_batch.cuh", "rsg_point.cuh",
+           "rsg_chain.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

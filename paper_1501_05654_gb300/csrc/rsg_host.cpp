@@ -757,7 +757,8 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
             cs = H->side;
             joined = false;
         }
-        CK(launch_proj_coeffs<R>(in, SV, H->pj, H->partial.as<double>(), H->pcnt.as<unsigned>(), h3, H->D.p, cs));
+        CK(launch_proj_coeffs<R>(in, SV, H->pj, H->partial.as<double>(), H->pcnt.as<unsigned>(), h3, H->D.p,
+                                 split_nl && joined, cs));
         if (!joined) CK(cudaEventRecord(H->ev_join, H->side));
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;

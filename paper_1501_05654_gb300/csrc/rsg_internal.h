@@ -156,9 +156,10 @@ inline int proj_slices(int SV) {
     const int bv = SV < 32 ? SV : 32;   // vector slices of the coefficient kernels: bv vectors each
     return (SV + bv - 1) / bv;
 }
+// chained: the launch may overlap the end of the kernel before it.
 template <typename R>
 cudaError_t launch_proj_coeffs(const void *u, int SV, const ProjDev &pj, double *partial, unsigned *counter,
-                               double h3, void *D, cudaStream_t st);
+                               double h3, void *D, bool chained, cudaStream_t st);
 template <typename R>
 cudaError_t launch_proj_dot(const void *u, int SV, const ProjDev &pj, double *partial,
                             cudaStream_t st);

@@ -31,6 +31,7 @@
 
 #include "rsg_async.cuh"
 #include "rsg_batch.cuh"
+#include "rsg_chain.cuh"
 #include "rsg_internal.h"
 #include "rsg_odd.cuh"
 #include "rsg_point.cuh"
@@ -516,11 +517,15 @@ __global__ void __launch_bounds__(kRowNT, 4) k_apply_row64(const ApplyArgs<R> a)
     static_assert(sizeof(R) == 8, "complex128");
     using V = VT<double>;
     __shared__ int4 nr[16];   // rows y-1, y+1, z-1, z+1, y-2, ...: start - xmin, xmin, xmax
+    chain_begin();
     const int row = blockIdx.x;
     const int ny = a.ny, SV = a.SV;
     const Row rc = a.rows[row];
     const int n = (rc.xmax - rc.xmin + 1) * SV;
-    if ((int)blockIdx.y * kRowNT >= n) return;
+    if ((int)blockIdx.y * kRowNT >= n) {
+        chain_wait();
+        return;
+    }
     const int z = row / ny, y = row - z * ny;
     if (threadIdx.x < 16) {
         const int k = (threadIdx.x >> 2) + 1, sgn = threadIdx.x & 1 ? k : -k;
@@ -528,6 +533,7 @@ __global__ void __launch_bounds__(kRowNT, 4) k_apply_row64(const ApplyArgs<R> a)
         nr[threadIdx.x] = make_int4(r.start - r.xmin, r.xmin, r.xmax, 0);
     }
     __syncthreads();
+    chain_wait();
     const double2 *__restrict__ in = (const double2 *)a.in;
     for (int t = blockIdx.y * kRowNT + threadIdx.x; t < n; t += gridDim.y * kRowNT) {
         const int xo = t / SV, v = t - xo * SV;
@@ -584,6 +590,7 @@ __global__ void __launch_bounds__(32 * kNaiveTY, 2) k_apply_naive(const ApplyArg
     __shared__ SRow rows[(kNaiveMaxZ + 8) * WY];
     // x range of each output row whose 16 in-plane neighbours all exist
     __shared__ int2 inner[kNaiveMaxZ * kNaiveTY];
+    chain_begin();
     const int ny = a.ny, nz = a.nz, SV = a.SV;
     const int y0 = blockIdx.y * kNaiveTY, z0 = blockIdx.z * zs;
     const int z1 = min(z0 + zs, nz);
@@ -604,6 +611,7 @@ __global__ void __launch_bounds__(32 * kNaiveTY, 2) k_apply_naive(const ApplyArg
         inner[i] = make_int2(lo, hi);
     }
     __syncthreads();
+    chain_wait();
     const int f = blockIdx.x * 32 + threadIdx.x;
     const int x = f / SV, v = f - x * SV, y = y0 + threadIdx.y;
     const bool lane_ok = x < a.nx && y < ny;
@@ -826,14 +834,15 @@ cudaError_t launch_apply(const ApplyArgs<R> &a, const TileCfg &cfg, int ntiles, 
         if constexpr (sizeof(R) == 8) {
             if (cfg.sum_zs > 0) return launch_apply_sum64(a, cfg.sum_zs, st);
             const long long per_row = ((long long)a.nx * a.SV + kRowNT - 1) / kRowNT;
-            k_apply_row64<R><<<dim3(a.ny * a.nz, (unsigned)(per_row < 65535 ? per_row : 65535)), kRowNT, 0, st>>>(a);
+            return launch_chained(k_apply_row64<R>, dim3(a.ny * a.nz, (unsigned)(per_row < 65535 ? per_row : 65535)),
+                                  dim3(kRowNT), 0, st, true, a);
         } else {
             const long long gx = ((long long)a.nx * a.SV + 31) / 32;
             if (gx > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
             const int gy = (a.ny + kNaiveTY - 1) / kNaiveTY, zs = naive_zs(gx * gy, a.nz);
-            k_apply_naive<R><<<dim3((unsigned)gx, gy, (a.nz + zs - 1) / zs), dim3(32, kNaiveTY), 0, st>>>(a, zs);
+            return launch_chained(k_apply_naive<R>, dim3((unsigned)gx, gy, (a.nz + zs - 1) / zs), dim3(32, kNaiveTY), 0, st,
+                                  true, a, zs);
         }
-        return cudaGetLastError();
     }
     if (ntiles == 0) return cudaSuccess;
     if (cfg.kernel == 2) {
@@ -901,6 +910,7 @@ __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__res
     static_assert(kDotChunk * NP * sizeof(R) <= sizeof(sm) && 2 * NP * 32 * V::NC * sizeof(double) <= sizeof(sm), "");
     R *qv = (R *)sm, *red = (R *)sm;
     double *cbuf = (double *)sm;   // c[i][s] of the slice (re, im)
+    chain_begin();
     const int c = blockIdx.x, bx = blockDim.x, by = blockDim.y;
     const int v = blockIdx.y * bx + threadIdx.x;
     const int tid = threadIdx.y * bx + threadIdx.x, nth = bx * by;
@@ -908,6 +918,7 @@ __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__res
     for (int i = tid; i < nq; i += nth) qs[i] = q_pt[q0 + i];
     for (int i = tid; i < nq * NP; i += nth) qv[i] = q_p[(int64_t)q0 * NP + i];
     __syncthreads();
+    chain_wait();
     T acc[NP];
 #pragma unroll
     for (int i = 0; i < NP; i++) acc[i] = V::zero();
@@ -999,12 +1010,12 @@ __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__res
 template <typename R>
 cudaError_t launch_proj_dot(const void *u, int SV, const ProjDev &pj, double *partial,
                             cudaStream_t st) {
-    return launch_proj_coeffs<R>(u, SV, pj, partial, nullptr, 0.0, nullptr, st);
+    return launch_proj_coeffs<R>(u, SV, pj, partial, nullptr, 0.0, nullptr, false, st);
 }
 
 template <typename R>
 cudaError_t launch_proj_coeffs(const void *u, int SV, const ProjDev &pj, double *partial, unsigned *counter,
-                               double h3, void *D, cudaStream_t st) {
+                               double h3, void *D, bool chained, cudaStream_t st) {
     if (pj.natoms == 0 || pj.nchunks == 0) return cudaSuccess;
     const int bv = SV < 32 ? SV : 32;
     const int pl = 256 / bv > 64 ? 64 : 256 / bv;
@@ -1014,17 +1025,16 @@ cudaError_t launch_proj_coeffs(const void *u, int SV, const ProjDev &pj, double 
     const T *uu = (const T *)u;
     const R *qp = (const R *)pj.q_p;
     R *DD = (R *)D;
-#define RSG_PROJ_DOT(NP_)                                                                                     \
-    k_proj_dot<R, NP_><<<grid, block, 0, st>>>(uu, SV, pj.q_pt, qp, pj.chunk_q0, pj.chunk_q1, partial, counter, \
-                                               pj.chunk_atom, pj.atom_chunk0, pj.hm, h3, DD)
+#define RSG_PROJ_DOT(NP_)                                                                                          \
+    return launch_chained(k_proj_dot<R, NP_>, grid, block, 0, st, chained, uu, SV, pj.q_pt, qp, pj.chunk_q0,          \
+                          pj.chunk_q1, partial, counter, pj.chunk_atom, pj.atom_chunk0, pj.hm, h3, DD)
     switch (pj.npmax) {
-    case 1: RSG_PROJ_DOT(1); break;
-    case 4: RSG_PROJ_DOT(4); break;
-    case 9: RSG_PROJ_DOT(9); break;
+    case 1: RSG_PROJ_DOT(1);
+    case 4: RSG_PROJ_DOT(4);
+    case 9: RSG_PROJ_DOT(9);
     default: return cudaErrorInvalidValue;
     }
 #undef RSG_PROJ_DOT
-    return cudaGetLastError();
 }
 
 // One thread per (atom, complex column s).  c_i = h3 * sum over the atom's
@@ -1079,6 +1089,7 @@ __global__ void __launch_bounds__(256) k_proj_scatter(const ApplyArgs<R> a, cons
                                                       const R *__restrict__ e_p, int nu) {
     using V = VT<R>;
     using T = typename V::T;
+    chain_begin();
     const int ub = blockIdx.x * blockDim.y * kScatPts + threadIdx.y;
     const T *D = (const T *)a.D;
     T *out = (T *)a.out;
@@ -2011,7 +2022,7 @@ template cudaError_t launch_apply<float>(const ApplyArgs<float> &, const TileCfg
 template cudaError_t launch_apply_naive_odd<float>(const ApplyArgs<float> &, cudaStream_t);
 template cudaError_t launch_proj_dot<float>(const void *, int, const ProjDev &, double *, cudaStream_t);
 template cudaError_t launch_proj_coeffs<float>(const void *, int, const ProjDev &, double *, unsigned *, double,
-                                               void *, cudaStream_t);
+                                               void *, bool, cudaStream_t);
 template cudaError_t launch_proj_reduce<float>(const double *, int, const ProjDev &, double, void *, cudaStream_t);
 template cudaError_t launch_proj_scatter<float>(const ApplyArgs<float> &, const ProjDev &, cudaStream_t);
 #endif
@@ -2022,7 +2033,7 @@ template cudaError_t launch_apply<double>(const ApplyArgs<double> &, const TileC
 template cudaError_t launch_apply_naive_odd<double>(const ApplyArgs<double> &, cudaStream_t);
 template cudaError_t launch_proj_dot<double>(const void *, int, const ProjDev &, double *, cudaStream_t);
 template cudaError_t launch_proj_coeffs<double>(const void *, int, const ProjDev &, double *, unsigned *, double,
-                                                void *, cudaStream_t);
+                                                void *, bool, cudaStream_t);
 template cudaError_t launch_proj_reduce<double>(const double *, int, const ProjDev &, double, void *, cudaStream_t);
 template cudaError_t launch_proj_scatter<double>(const ApplyArgs<double> &, const ProjDev &, cudaStream_t);
 #endif

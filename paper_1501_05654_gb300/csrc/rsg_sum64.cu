@@ -30,6 +30,7 @@
 // against 80-bit sums on noise, packets and values spread over 2^+-900, of
 // the norm: 1.35e-16, 9.8e-16, 1.1e-16 (FP64 sums 1.39e-16, 1.1e-15, 1.1e-16).
 #include "rsg_async.cuh"
+#include "rsg_chain.cuh"
 #include "rsg_internal.h"
 #include "rsg_point.cuh"
 #include "rsg_vec.cuh"
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(kSumNT, 2) k_apply_sum64(const ApplyArgs<doubl
     __shared__ longlong2 wm[2][WY * WX * NSC];
     __shared__ int we[2][WY * WX * NSC];
     __shared__ SRow rows[(kSumMaxZ + 8) * WY];
+    chain_begin();
     const int ny = a.ny, nz = a.nz, SV = a.SV;
     const int ntx = (a.nx + TX - 1) / TX;
     const int tile = blockIdx.x / nch, s0 = (blockIdx.x - tile * nch) * NSC;
@@ -122,7 +124,9 @@ __global__ void __launch_bounds__(kSumNT, 2) k_apply_sum64(const ApplyArgs<doubl
         rows[i] = SRow{r.start - r.xmin, (int16_t)r.xmin, (int16_t)r.xmax};
         any = any || (wy >= 4 && wy < WY - 4 && zz >= z0 && zz < z1 && r.xmin < x0 + TX && r.xmax >= x0);
     }
-    if (!__syncthreads_or(any)) return;
+    any = __syncthreads_or(any);
+    chain_wait();
+    if (!any) return;
     const bool vok = v < SV;
     const double2 *__restrict__ in = (const double2 *)a.in;
     auto value = [&](const SRow &r, int xx, int vv) -> double2 {
@@ -272,9 +276,8 @@ cudaError_t launch_apply_sum64(const ApplyArgs<double> &a, int zs, cudaStream_t 
     const long long nb = (long long)((a.nx + tx - 1) / tx) * ((a.ny + ty - 1) / ty) * nch;
     if (nb > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const dim3 grid((unsigned)nb, (a.nz + zs - 1) / zs);
-    if (nsc == 1) k_apply_sum64<1><<<grid, kSumNT, 0, st>>>(a, zs, (int)nch);
-    else k_apply_sum64<2><<<grid, kSumNT, 0, st>>>(a, zs, (int)nch);
-    return cudaGetLastError();
+    return launch_chained(nsc == 1 ? k_apply_sum64<1> : k_apply_sum64<2>, grid, dim3(kSumNT), 0, st, true, a, zs,
+                          (int)nch);
 }
 
 }  // namespace rsg

@@ -43,6 +43,7 @@
 #include <unordered_map>
 
 #include "rsg_async.cuh"
+#include "rsg_chain.cuh"
 #include "rsg_internal.h"
 #include "rsg_vec.cuh"
 
@@ -126,6 +127,7 @@ __global__ void __launch_bounds__(WideGeom<NYP, NPW>::NT, 1)
     k_apply_wide(const ApplyArgs<float> a, int nchunks, const __grid_constant__ WideMaps maps) {
     using G = WideGeom<NYP, NPW>;
     constexpr int TX = G::TX, TY = G::TY, WX = G::WX, WY = G::WY, NC = G::NC, NCW = G::NCW;
+    chain_begin();
     extern __shared__ __align__(128) unsigned char smraw[];
     // 1024-byte aligned start: u ring, base ring, potential ring, row table,
     // barriers, abort flag
@@ -199,6 +201,7 @@ __global__ void __launch_bounds__(WideGeom<NYP, NPW>::NT, 1)
     }
     jf = __reduce_min_sync(0xffffffffu, jf);
     jl = __reduce_max_sync(0xffffffffu, jl);
+    chain_wait();
     if (jl < 0) return;
     const int j0 = jf, j1 = min(np - 1, jl + 4);
     if (tid == 0) {
@@ -570,9 +573,8 @@ static cudaError_t launch_wide_t(const ApplyArgs<float> &a, const TileCfg &cfg, 
     const int nchunks = (ld + G::NC - 1) / G::NC;
     const long long nblk = (long long)ntiles * nchunks;
     if (nblk > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    kern<<<(unsigned)nblk, G::NT, smem, st>>>(a, nchunks, maps);
     *launched = true;
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)nblk), dim3(G::NT), smem, st, true, a, nchunks, maps);
 }
 
 cudaError_t launch_apply_wide(const ApplyArgs<float> &a, const TileCfg &cfg, int ntiles, cudaStream_t st,
