@@ -513,20 +513,38 @@ TileCfg choose_c64(rsg_ham H, int SV) {
     const int nch7 = (SV + 7) / 8, nch5 = (SV + 1) / 2;
     const bool nl = H->pj.natoms > 0;
     int64_t n = 0;
-    makespan(col7, best.zseg, nch7, 152, &n);
-    if (SV % 8 != 0 || n < 4 * 152) {
-        const double vec = (double)m->P * SV, tiled = nl ? 8.0 : 2.0;
-        double cost = H->has_scaling ? 10.0 + 40e-6 * vec : (5.0 + 30e-6 * vec) * (nl ? 1.2 : 1.0);
+    const double vec = (double)m->P * SV, tiled = nl ? 8.0 : 2.0;
+    const double plain = H->has_scaling ? 10.0 + 40e-6 * vec : (5.0 + 30e-6 * vec) * (nl ? 1.2 : 1.0);
+    auto time7 = [&](int zs) { return tiled + 0.97 * makespan(col7, zs, nch7, 152, &n); };
+    auto time5 = [&](int zs) {
+        const double mk = makespan(col5, zs, nch5, 304, &n);
+        return tiled + (n <= 152 ? 0.92 : 1.2) * mk;
+    };
+    // without a cut: kernel 7, kernel 5 for narrow rows with a partly empty
+    // chunk, the plain kernel where that leaves SMs without a block
+    const bool narrow = SV % 8 != 0 && SV < 20;
+    double cost = narrow ? time5(150) : time7(best.zseg);
+    if (narrow) {
+        best = c5;
+        best.zseg = 150;
+    }
+    if (n < (narrow ? 304 : 152)) {
         best.kernel = 1;
+        cost = plain;
+    }
+    if (narrow || n < 4 * 152) {
+        cost *= 0.92;   // the fit is good to a few percent: change for a clear gain only
+        if (plain < cost) {
+            cost = plain;
+            best.kernel = 1;
+        }
         for (int zs : {190, 150, 96, 64, 48, 32, 24, 16, 12, 8}) {
-            const double m7 = makespan(col7, zs, nch7, 152, &n);
-            if (tiled + 0.97 * m7 < cost) {
-                cost = tiled + 0.97 * m7;
+            const double t7 = time7(zs), t5 = time5(zs);
+            if (t7 < cost) {
+                cost = t7;
                 best = H->cfg;
                 best.zseg = zs;
             }
-            const double m5 = makespan(col5, zs, nch5, 304, &n);
-            const double t5 = tiled + (n <= 152 ? 0.92 : 1.2) * m5;
             if (zs <= 150 && t5 < cost) {
                 cost = t5;
                 best = c5;
@@ -554,7 +572,7 @@ int choose_c128(rsg_ham H, int SV) {
     const int ns = sum64_states(SV), nch = (SV + ns - 1) / ns;
     TileCfg best = H->cfg;
     best.sum_zs = 0;
-    double cost = 6.0 + 125e-6 * (double)H->m->P * SV;
+    double cost = 0.95 * (6.0 + 125e-6 * (double)H->m->P * SV);
     for (int zs : {32, 24, 16, 12, 8, 6, 4, 3, 2, 1}) {
         int64_t n = 0;
         const double mk = makespan(col, zs, nch, 152, &n, 5, 1);
