@@ -1078,11 +1078,14 @@ __global__ void k_proj_reduce(const double *__restrict__ partial, int SV, int na
 //     acc[p, v] += gamma * alpha * (same)            (when acc is used)
 // one thread per (union point, vector); the union points and their entry
 // lists come from the point-centric CSR, so there are no atomics.
-// Each block row (threadIdx.y) takes kScatPts union points, blockDim.y rows
-// apart; their index, state and first-entry loads are issued before any of
-// them is used, so that several points' loads are in flight per warp.
+// Each block row (threadIdx.y) takes kScatPts neighbouring union points; their
+// index, state and first-entry loads are issued before any of them is used, so
+// that several points' loads are in flight per warp.  Neighbouring points
+// mostly lie in the same sphere: where all of a row's points have one entry of
+// one atom, each coefficient is read once for them (192^3, 64 atoms x 9, 128
+// states: the coefficients are 9 KB a point, the states 2 KB).
 constexpr int kScatPts = 4;
-template <typename R>
+template <typename R, int NP>
 __global__ void __launch_bounds__(256) k_proj_scatter(const ApplyArgs<R> a, const int32_t *__restrict__ upts,
                                                       const int32_t *__restrict__ uptr,
                                                       const int32_t *__restrict__ e_atom,
@@ -1090,36 +1093,55 @@ __global__ void __launch_bounds__(256) k_proj_scatter(const ApplyArgs<R> a, cons
     using V = VT<R>;
     using T = typename V::T;
     chain_begin();
-    const int ub = blockIdx.x * blockDim.y * kScatPts + threadIdx.y;
+    const int ub = (blockIdx.x * blockDim.y + threadIdx.y) * kScatPts;
     const T *D = (const T *)a.D;
     T *out = (T *)a.out;
     int p[kScatPts], e0[kScatPts], e1[kScatPts], at0[kScatPts];
 #pragma unroll
     for (int k = 0; k < kScatPts; k++) {
-        const int u = ub + k * (int)blockDim.y;
+        const int u = ub + k;
         const bool ok = u < nu;
         p[k] = ok ? upts[u] : -1;
         e0[k] = ok ? uptr[u] : 0;
         e1[k] = ok ? uptr[u + 1] : 0;
     }
+    bool one = p[kScatPts - 1] >= 0;   // every point exists, with one entry of the same atom
 #pragma unroll
     for (int k = 0; k < kScatPts; k++) at0[k] = e1[k] > e0[k] ? e_atom[e0[k]] : 0;
-    for (int v = threadIdx.x; v < a.SV; v += blockDim.x) {
-        T o[kScatPts];
 #pragma unroll
-        for (int k = 0; k < kScatPts; k++) o[k] = p[k] >= 0 ? out[(int64_t)p[k] * a.SV + v] : V::zero();
+    for (int k = 0; k < kScatPts; k++) one = one && e1[k] == e0[k] + 1 && at0[k] == at0[0];
+    for (int v = threadIdx.x; v < a.SV; v += blockDim.x) {
+        T o[kScatPts], sum[kScatPts];
+#pragma unroll
+        for (int k = 0; k < kScatPts; k++) {
+            o[k] = p[k] >= 0 ? out[(int64_t)p[k] * a.SV + v] : V::zero();
+            sum[k] = V::zero();
+        }
+        if (one) {
+            const T *Da = D + (int64_t)at0[0] * NP * a.SV + v;
+            const R *pv = e_p + (int64_t)e0[0] * NP;   // the points' entries follow each other
+#pragma unroll
+            for (int i = 0; i < NP; i++) {
+                const T d = Da[(int64_t)i * a.SV];
+#pragma unroll
+                for (int k = 0; k < kScatPts; k++) V::fma(sum[k], pv[k * NP + i], d);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < kScatPts; k++)
+                for (int e = e0[k]; e < e1[k]; e++) {
+                    const int at = e == e0[k] ? at0[k] : e_atom[e];
+                    const R *pv = e_p + (int64_t)e * NP;
+                    const T *Da = D + (int64_t)at * NP * a.SV + v;
+#pragma unroll
+                    for (int i = 0; i < NP; i++) V::fma(sum[k], pv[i], Da[(int64_t)i * a.SV]);
+                }
+        }
 #pragma unroll
         for (int k = 0; k < kScatPts; k++) {
             if (p[k] < 0) continue;
-            T sum = V::zero();
-            for (int e = e0[k]; e < e1[k]; e++) {
-                const int at = e == e0[k] ? at0[k] : e_atom[e];
-                const R *pv = e_p + (int64_t)e * a.npmax;
-                const T *Da = D + (int64_t)at * a.npmax * a.SV + v;
-                for (int i = 0; i < a.npmax; i++) V::fma(sum, pv[i], Da[(int64_t)i * a.SV]);
-            }
             const int64_t oi = (int64_t)p[k] * a.SV + v;
-            const T y = V::cmul(a.ar, a.ai, sum);
+            const T y = V::cmul(a.ar, a.ai, sum[k]);
             out[oi] = V::add(o[k], y);
             if (a.acc != nullptr) {
                 T sacc = ((T *)a.acc)[oi];
@@ -1137,8 +1159,16 @@ cudaError_t launch_proj_scatter(const ApplyArgs<R> &a, const ProjDev &pj, cudaSt
     const int bx = a.SV < 32 ? a.SV : 32;
     const int by = 256 / bx;
     const int per = by * kScatPts;
-    k_proj_scatter<R><<<(nu + per - 1) / per, dim3(bx, by), 0, st>>>(a, pj.u_pts, pj.u_ptr, pj.e_atom,
-                                                                    (const R *)pj.e_p, nu);
+#define RSG_PROJ_SCATTER(NP_)                                                                                    \
+    k_proj_scatter<R, NP_><<<(nu + per - 1) / per, dim3(bx, by), 0, st>>>(a, pj.u_pts, pj.u_ptr, pj.e_atom,       \
+                                                                         (const R *)pj.e_p, nu)
+    switch (pj.npmax) {
+    case 1: RSG_PROJ_SCATTER(1); break;
+    case 4: RSG_PROJ_SCATTER(4); break;
+    case 9: RSG_PROJ_SCATTER(9); break;
+    default: return cudaErrorInvalidValue;
+    }
+#undef RSG_PROJ_SCATTER
     return cudaGetLastError();
 }
 
