@@ -2316,7 +2316,8 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
         for (int d = 0; d < 3; d++) H->xdir_cached[d] = dir[d];
     }
     const int nb = norm_blocks(P);
-    CK(H->dots.ensure((size_t)nb * 20 * sizeof(double) + 64 * sizeof(double)));
+    const int nba = adjoint_blocks(P);
+    CK(H->dots.ensure((size_t)std::max(20 * nb, nba) * sizeof(double) + 64 * sizeof(double)));
     CK(H->M.ensure(32 * sizeof(double)));
     CK(H->ov.ensure(2 * sizeof(double)));
     CK(H->grad.ensure((size_t)nsteps * sizeof(double) + 64));
@@ -2438,7 +2439,7 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
                         bb[j] = (const char *)arr(br, t, j) + cb;
                         aa[j] = arr(bc, tc, j);
                     }
-                    CK(launch_adjoint_grad<R>(bb, aa, P, 2, H->Xd.as<R>(), h3, tau, H->dots.as<double>(), nb,
+                    CK(launch_adjoint_grad<R>(bb, aa, P, 2, H->Xd.as<R>(), h3, tau, H->dots.as<double>(), nba,
                                               counter, H->grad.as<double>() + k, st));
                 }
             }
@@ -2473,7 +2474,7 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
                 const void *aa[4] = {a0, keep_powers ? pslot(k - k0, l, 1) : pslot(0, l, 1),
                                      keep_powers ? pslot(k - k0, l, 2) : pslot(0, l, 2),
                                      keep_powers ? pslot(k - k0, l, 3) : pslot(0, l, 3)};
-                CK(launch_adjoint_grad<R>(bb, aa, P, (int)ld, H->Xd.as<R>(), h3, tau, H->dots.as<double>(), nb,
+                CK(launch_adjoint_grad<R>(bb, aa, P, (int)ld, H->Xd.as<R>(), h3, tau, H->dots.as<double>(), nba,
                                           counter, H->grad.as<double>() + k, st));
                 std::swap(chi, chi2);
             }

@@ -239,6 +239,7 @@ template <typename R>
 cudaError_t launch_adjoint_grad(const void *const *b, const void *const *a, int64_t P, int ld,
                                 const R *X, double h3, double tau, double *partial, int nblk,
                                 unsigned *counter, double *grad_k, cudaStream_t st);
+int adjoint_blocks(int64_t P);   // nblk of launch_adjoint_grad
 // overlap: out = h3 sum_p conj(f_p) g_p  (complex double, one state)
 template <typename R>
 cudaError_t launch_overlap(const void *f, const void *g, int64_t P, int ld, double h3,

@@ -10,6 +10,7 @@
 // FP64 reductions as well.
 #include <algorithm>
 
+#include "rsg_chain.cuh"
 #include "rsg_internal.h"
 #include "rsg_vec.cuh"
 
@@ -403,13 +404,14 @@ __global__ void __launch_bounds__(256) k_adjoint_grad(const R *b0, const R *b1, 
     const int64_t p1 = p0 + per < P ? p0 + per : P;
     constexpr double f2 = 0.5, f3 = 1.0 / 6.0, f4 = 1.0 / 24.0;
     double acc = 0.0;
+    chain_begin();
+    chain_wait();
     for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
         const int64_t o = p * ld * 2;
-        double br0, bi0, br1, bi1, br2, bi2, br3, bi3, ar, ai;
-        ld_c(b0 + o, br0, bi0);
-        ld_c(b1 + o, br1, bi1);
-        ld_c(b2 + o, br2, bi2);
-        ld_c(b3 + o, br3, bi3);
+        const double br0 = widen(b0[o]), bi0 = widen(b0[o + 1]), br1 = widen(b1[o]), bi1 = widen(b1[o + 1]);
+        const double br2 = widen(b2[o]), bi2 = widen(b2[o + 1]), br3 = widen(b3[o]), bi3 = widen(b3[o + 1]);
+        const double ar0 = widen(a0[o]), ai0 = widen(a0[o + 1]), ar1 = widen(a1[o]), ai1 = widen(a1[o + 1]);
+        const double ar2 = widen(a2[o]), ai2 = widen(a2[o + 1]), ar3 = widen(a3[o]), ai3 = widen(a3[o + 1]);
         // c_0 .. c_3
         const double c0r = fma(f4, br3, fma(f3, br2, fma(f2, br1, br0)));
         const double c0i = fma(f4, bi3, fma(f3, bi2, fma(f2, bi1, bi0)));
@@ -418,15 +420,11 @@ __global__ void __launch_bounds__(256) k_adjoint_grad(const R *b0, const R *b1, 
         const double c2r = fma(f4, br1, f3 * br0), c2i = fma(f4, bi1, f3 * bi0);
         const double c3r = f4 * br0, c3i = f4 * bi0;
         double t;
-        ld_c(a0 + o, ar, ai);
-        t = fma(c0r, ai, -c0i * ar);
-        ld_c(a1 + o, ar, ai);
-        t = fma(c1r, ai, fma(-c1i, ar, t));
-        ld_c(a2 + o, ar, ai);
-        t = fma(c2r, ai, fma(-c2i, ar, t));
-        ld_c(a3 + o, ar, ai);
-        t = fma(c3r, ai, fma(-c3i, ar, t));
-        acc = fma((double)X[p], t, acc);
+        t = fma(c0r, ai0, -c0i * ar0);
+        t = fma(c1r, ai1, fma(-c1i, ar1, t));
+        t = fma(c2r, ai2, fma(-c2i, ar2, t));
+        t = fma(c3r, ai3, fma(-c3i, ar3, t));
+        acc = fma(widen(X[p]), t, acc);
     }
     // block sum: shuffles within each warp, then the warps in order
 #pragma unroll
@@ -459,14 +457,17 @@ __global__ void __launch_bounds__(256) k_adjoint_grad(const R *b0, const R *b1, 
     *counter = 0u;
 }
 
+// Four blocks per SM: 28 FP64 instructions a point (two a clock per SM) need
+// every SM; one block per 2048 points left 24 of them idle at 64^3.
+int adjoint_blocks(int64_t P) { return (int)std::max<int64_t>(1, std::min<int64_t>(608, (P + 255) / 256)); }
+
 template <typename R>
 cudaError_t launch_adjoint_grad(const void *const *b, const void *const *a, int64_t P, int ld, const R *X,
                                 double h3, double tau, double *partial, int nblk, unsigned *counter,
                                 double *grad_k, cudaStream_t st) {
-    k_adjoint_grad<R><<<nblk, 256, 0, st>>>((const R *)b[0], (const R *)b[1], (const R *)b[2], (const R *)b[3],
-                                            (const R *)a[0], (const R *)a[1], (const R *)a[2], (const R *)a[3], P,
-                                            ld, X, h3, tau, partial, nblk, counter, grad_k);
-    return cudaGetLastError();
+    return launch_chained(k_adjoint_grad<R>, dim3(nblk), dim3(256), 0, st, true, (const R *)b[0], (const R *)b[1],
+                          (const R *)b[2], (const R *)b[3], (const R *)a[0], (const R *)a[1], (const R *)a[2],
+                          (const R *)a[3], P, ld, X, h3, tau, partial, nblk, counter, grad_k);
 }
 
 // Expand the 10 packed values into out[j*4+i] (complex double), zero elsewhere.
