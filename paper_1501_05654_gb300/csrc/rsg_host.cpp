@@ -438,11 +438,17 @@ const std::vector<int> &column_lengths(rsg_mesh m, int TX, int TY) {
     const int ntx = (m->nx + TX - 1) / TX, nty = (m->ny + TY - 1) / TY;
     std::vector<int> zlo((size_t)ntx * nty, m->nz), zhi((size_t)ntx * nty, 0);
     for (int z = 0; z < m->nz; z++)
-        for (int y = 0; y < m->ny; y++) {
-            const Row &r = m->rows[(size_t)z * m->ny + y];
-            if (r.xmin > r.xmax) continue;
-            for (int tx = r.xmin / TX; tx <= r.xmax / TX; tx++) {
-                const size_t k = (size_t)(y / TY) * ntx + tx;
+        for (int ty = 0; ty < nty; ty++) {
+            // the tile's rows together (every shape is convex)
+            int lo = m->nx, hi = -1;
+            for (int y = ty * TY; y < std::min(m->ny, (ty + 1) * TY); y++) {
+                const Row &r = m->rows[(size_t)z * m->ny + y];
+                if (r.xmin > r.xmax) continue;
+                lo = std::min(lo, r.xmin);
+                hi = std::max(hi, r.xmax);
+            }
+            for (int tx = lo / TX; tx <= (hi < 0 ? -1 : hi / TX); tx++) {
+                const size_t k = (size_t)ty * ntx + tx;
                 zlo[k] = std::min(zlo[k], z);
                 zhi[k] = z + 1;
             }
@@ -456,30 +462,47 @@ const std::vector<int> &column_lengths(rsg_mesh m, int TX, int TY) {
 
 // Time until the last of `slots` resident blocks is done: columns cut into
 // segments of zs planes, nch blocks per segment that take mul * planes + add,
-// longest first to the first free slot; *blocks receives their number.
-double makespan(const std::vector<int> &col, int zs, int nch, int slots, int64_t *blocks, int mul = 1, int add = 8) {
-    std::map<int, int64_t, std::greater<int>> by_len;   // time -> blocks
-    int64_t n = 0, total = 0;
-    for (int L : col)
-        for (int z = 0; z < L; z += zs) {
-            const int len = mul * std::min(zs, L - z) + add;
-            by_len[len] += nch;
-            n += nch;
-            total += (int64_t)len * nch;
-        }
+// longest first to the first free slot; *blocks receives their number.  A
+// schedule whose load alone takes `enough` is not worked out.
+double makespan(const std::vector<int> &col, int zs, int nch, int slots, int64_t *blocks, int mul = 1, int add = 8,
+                double enough = 1e300) {
+    // blocks by planes, rounded up to a sixteenth of the longest
+    const int longest = col.empty() ? 0 : std::min(zs, col[0]), step = longest / 16 + 1;
+    std::vector<int64_t> by_len((size_t)(longest / step + 2), 0);
+    int64_t n = 0;
+    for (int L : col) {
+        const int full = L / zs, rest = L % zs;
+        if (full) by_len[(size_t)((zs + step - 1) / step)] += (int64_t)full * nch;
+        if (rest) by_len[(size_t)((rest + step - 1) / step)] += nch;
+        n += (int64_t)(full + (rest > 0)) * nch;
+    }
     *blocks = n;
     if (n == 0) return 0.0;
-    if (n > 16 * (int64_t)slots) return (double)total / slots + 0.5 * by_len.begin()->first;
-    std::vector<int64_t> heap((size_t)slots, 0);   // min-heap of finish times
-    int64_t last = 0;
-    for (const auto &b : by_len)
-        for (int64_t k = 0; k < b.second; k++) {
-            std::pop_heap(heap.begin(), heap.end(), std::greater<int64_t>());
-            heap.back() += b.first;
-            last = std::max(last, heap.back());
-            std::push_heap(heap.begin(), heap.end(), std::greater<int64_t>());
+    double load = 0.0;
+    for (size_t k = 0; k < by_len.size(); k++)
+        load += (double)by_len[k] * ((double)mul * std::min<int64_t>((int64_t)k * step, longest) + add);
+    if (load / slots >= enough) return load / slots;
+    // finish times of the slots and how many slots finish at each
+    std::map<int64_t, int64_t> at{{0, slots}};
+    for (size_t k = by_len.size(); k-- > 0;) {
+        const int64_t len = (int64_t)mul * std::min<int64_t>((int64_t)k * step, longest) + add;
+        int64_t left = by_len[k];
+        if (left >= 4 * (int64_t)slots) {   // whole rounds keep the order of the finish times
+            const int64_t rounds = left / slots - 2;
+            std::map<int64_t, int64_t> moved;
+            for (const auto &t : at) moved[t.first + rounds * len] = t.second;
+            at.swap(moved);
+            left -= rounds * slots;
         }
-    return (double)last;
+        while (left > 0) {
+            const auto it = at.begin();
+            const int64_t t = it->first, take = std::min(left, it->second);
+            if ((it->second -= take) == 0) at.erase(it);
+            at[t + len] += take;
+            left -= take;
+        }
+    }
+    return (double)at.rbegin()->first;
 }
 
 // Stencil kernel and segment length of the default complex64 configuration.
@@ -506,23 +529,32 @@ TileCfg choose_c64(rsg_ham H, int SV) {
     c5.threads = 192;
     c5.stages = 3;
     c5.sync = 0;
+    const int nch7 = (SV + 7) / 8, nch5 = (SV + 1) / 2;
+    const bool narrow = SV % 8 != 0 && SV < 20, nl = H->pj.natoms > 0;
     int tx7, ty7, tx5, ty5;
     block_shape(H->cfg, SV, &tx7, &ty7);
     block_shape(c5, SV, &tx5, &ty5);
-    const std::vector<int> &col7 = column_lengths(m, tx7, ty7), &col5 = column_lengths(m, tx5, ty5);
-    const int nch7 = (SV + 7) / 8, nch5 = (SV + 1) / 2;
-    const bool nl = H->pj.natoms > 0;
+    if (!narrow) {
+        // enough blocks without a cut: nothing to choose
+        const Tile *tiles = nullptr;
+        int nt = 0;
+        if (get_tiles(m, tx7, ty7, best.zseg, &tiles, &nt) != RSG_OK || (int64_t)nt * nch7 >= 4 * 152)
+            return H->auto_cfg[key] = best;
+    }
+    const std::vector<int> &col7 = column_lengths(m, tx7, ty7), none;
+    const std::vector<int> &col5 = SV % 8 != 0 ? column_lengths(m, tx5, ty5) : none;
     int64_t n = 0;
     const double vec = (double)m->P * SV, tiled = nl ? 8.0 : 2.0;
     const double plain = H->has_scaling ? 10.0 + 40e-6 * vec : (5.0 + 30e-6 * vec) * (nl ? 1.2 : 1.0);
-    auto time7 = [&](int zs) { return tiled + 0.97 * makespan(col7, zs, nch7, 152, &n); };
-    auto time5 = [&](int zs) {
-        const double mk = makespan(col5, zs, nch5, 304, &n);
+    auto time7 = [&](int zs, double enough = 1e300) {
+        return tiled + 0.97 * makespan(col7, zs, nch7, 152, &n, 1, 8, (enough - tiled) / 0.97);
+    };
+    auto time5 = [&](int zs, double enough = 1e300) {
+        const double mk = makespan(col5, zs, nch5, 304, &n, 1, 8, (enough - tiled) / 0.92);
         return tiled + (n <= 152 ? 0.92 : 1.2) * mk;
     };
     // without a cut: kernel 7, kernel 5 for narrow rows with a partly empty
     // chunk, the plain kernel where that leaves SMs without a block
-    const bool narrow = SV % 8 != 0 && SV < 20;
     double cost = narrow ? time5(150) : time7(best.zseg);
     if (narrow) {
         best = c5;
@@ -532,24 +564,26 @@ TileCfg choose_c64(rsg_ham H, int SV) {
         best.kernel = 1;
         cost = plain;
     }
-    if (narrow || n < 4 * 152) {
-        cost *= 0.92;   // the fit is good to a few percent: change for a clear gain only
-        if (plain < cost) {
-            cost = plain;
-            best.kernel = 1;
+    cost *= 0.92;   // the fit is good to a few percent: change for a clear gain only
+    if (plain < cost) {
+        cost = plain;
+        best.kernel = 1;
+    }
+    int last = 0;
+    for (int zs : {190, 150, 96, 64, 48, 32, 24, 16, 12, 8}) {
+        if (!col7.empty() && zs >= col7[0] && last >= col7[0]) continue;   // no cut either way
+        last = zs;
+        const double t7 = time7(zs, cost);
+        if (t7 < cost) {
+            cost = t7;
+            best = H->cfg;
+            best.zseg = zs;
         }
-        for (int zs : {190, 150, 96, 64, 48, 32, 24, 16, 12, 8}) {
-            const double t7 = time7(zs), t5 = time5(zs);
-            if (t7 < cost) {
-                cost = t7;
-                best = H->cfg;
-                best.zseg = zs;
-            }
-            if (zs <= 150 && t5 < cost) {
-                cost = t5;
-                best = c5;
-                best.zseg = zs;
-            }
+        const double t5 = SV % 8 != 0 && zs <= 150 ? time5(zs, cost) : cost;
+        if (t5 < cost) {
+            cost = t5;
+            best = c5;
+            best.zseg = zs;
         }
     }
     return H->auto_cfg[key] = best;
@@ -575,7 +609,7 @@ int choose_c128(rsg_ham H, int SV) {
     double cost = 0.95 * (6.0 + 125e-6 * (double)H->m->P * SV);
     for (int zs : {32, 24, 16, 12, 8, 6, 4, 3, 2, 1}) {
         int64_t n = 0;
-        const double mk = makespan(col, zs, nch, 152, &n, 5, 1);
+        const double mk = makespan(col, zs, nch, 152, &n, 5, 1, (cost - 3.0) / (2.55 / 5));
         const double t = 3.0 + std::max(2.55 / 5 * mk, 3.2 * (col.empty() ? 0 : std::min(zs, col[0])));
         if (t < cost) {
             cost = t;
