@@ -2199,21 +2199,24 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
         CK(cudaStreamSynchronize(st));
         return RSG_OK;
     };
-    auto upload = [&](const std::vector<std::complex<double>> &v, double *dst) -> rsg_status {
+    // dst = v and, with neg, -v behind it (d_a, d_b). The copy is not waited for:
+    // coef is written again only after a stream sync, mostly that of a reduction's
+    // download, which every pair of uploads has between them.
+    auto upload = [&](const std::vector<std::complex<double>> &v, double *dst, bool neg) -> rsg_status {
         for (int64_t s = 0; s < S; s++) {
             coef[(size_t)2 * s] = v[(size_t)s].real();
             coef[(size_t)2 * s + 1] = v[(size_t)s].imag();
+            coef[(size_t)(2 * (S + s))] = -v[(size_t)s].real();
+            coef[(size_t)(2 * (S + s)) + 1] = -v[(size_t)s].imag();
         }
-        CK(cudaMemcpyAsync(dst, coef.data(), (size_t)2 * S * sizeof(double), cudaMemcpyHostToDevice, st));
-        CK(cudaStreamSynchronize(st));     // coef is reused by the next upload
+        CK(cudaMemcpyAsync(dst, coef.data(), (size_t)(neg ? 4 : 2) * S * sizeof(double), cudaMemcpyHostToDevice, st));
         return RSG_OK;
     };
     using cd = std::complex<double>;
-    std::vector<cd> rho((size_t)S), mu((size_t)S), alpha((size_t)S), beta((size_t)S), neg((size_t)S);
+    std::vector<cd> rho((size_t)S), mu((size_t)S), alpha((size_t)S), beta((size_t)S), minus((size_t)S, -1.0);
     // r = b - A x, p = r
     CKS(Ax(x, q));
-    for (int64_t s = 0; s < S; s++) neg[(size_t)s] = -1.0;
-    CKS(upload(neg, d_a));
+    CKS(upload(minus, d_a, false));
     CKS(comb(b, q, r, d_a));
     CK(cudaMemcpyAsync(p, r, bytes, cudaMemcpyDeviceToDevice, st));
     CKS(norms(b, bn));
@@ -2243,11 +2246,9 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
                     return fail(RSG_ERR_NONFINITE, "breakdown: p^T (H - z) p = 0 for state %lld", (long long)s);
                 alpha[(size_t)s] = rho[(size_t)s] / mu[(size_t)s];
             }
-            neg[(size_t)s] = -alpha[(size_t)s];
         }
-        CKS(upload(alpha, d_a));
+        CKS(upload(alpha, d_a, true));
         CKS(comb(x, p, x, d_a));          // x += alpha p
-        CKS(upload(neg, d_b));
         CKS(comb(r, q, r, d_b));          // r -= alpha q
         CKS(bilinear(r, r));
         CKS(norms(r, nrm));
@@ -2256,14 +2257,14 @@ rsg_status rsg_shifted_solve(rsg_ham H, const void *b, void *x, int64_t S, int64
             beta[(size_t)s] = done[(size_t)s] || std::abs(rho[(size_t)s]) == 0.0 ? cd(0.0) : rn / rho[(size_t)s];
             rho[(size_t)s] = rn;
         }
-        CKS(upload(beta, d_b));
+        CKS(upload(beta, d_b, false));
         CKS(comb(r, p, p, d_b));          // p = r + beta p
         it++;
     }
     // true residual |b - (H - z) x| / |b|
     CKS(Ax(x, q));
-    for (int64_t s = 0; s < S; s++) neg[(size_t)s] = -1.0;
-    CKS(upload(neg, d_a));
+    CK(cudaStreamSynchronize(st));        // the last beta may still be in coef
+    CKS(upload(minus, d_a, false));
     CKS(comb(b, q, r, d_a));
     CKS(norms(r, nrm));
     if (resid_out)

@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(1024) k_sum_rows(const double *__restrict__ pa
         v = load(b0 + 32);
         if (threadIdx.y == 0) {
             const int m = min(32, nblk - b0);
+#pragma unroll 8
             for (int q = 0; q < m; q++) s += buf[k][q][threadIdx.x];
         }
     }
