@@ -2400,7 +2400,10 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
     // their Hamiltonian applications runs as one two-column launch: column 0
     // the recompute (A = -i tau H(eps_r)), column 1 the costate
     // (A^dagger = +i tau H(eps_c)).  Two banks of two-column blocks hold the
-    // powers of consecutive segments.
+    // powers of consecutive segments.  The last segment's recompute and the
+    // first segment's costate have no partner: their bank's blocks are one
+    // state wide (ld = 1; complex64 rows are two values wide anyway), where a
+    // complex128 application costs half of a two-column one.
     const size_t vb2 = (size_t)P * 2 * cb;
     const int64_t nper = (int64_t)K * m * 4 + 1;     // per bank: 4 powers of every step, and the segment's end
     const bool merged = keep_powers && (H->adj_merge == 1 ||
@@ -2410,16 +2413,16 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
         for (int64_t i = 0; i < 2 * nper + 1; i++) CK(H->pool2[(size_t)i].ensure(vb2));
         auto arr = [&](int b, int64_t t, int j) { return H->pool2[(size_t)(b * nper + t * 4 + j)].p; };
         void *scr = H->pool2[(size_t)(2 * nper)].p;
-        // column col of a two-column block <-> a single-state vector
-        auto to_col = [&](void *blk, int col, const void *v) {
-            return cudaMemcpy2DAsync((char *)blk + col * cb, 2 * cb, v, ld * cb, cb, (size_t)P,
+        int64_t width[2] = {2, 2};   // columns of each bank's blocks; the costate is the last
+        // column col of a bank's block <-> a single-state vector
+        auto to_col = [&](int b, void *blk, int64_t col, const void *v) {
+            return cudaMemcpy2DAsync((char *)blk + col * cb, width[b] * cb, v, ld * cb, cb, (size_t)P,
                                      cudaMemcpyDeviceToDevice, st);
         };
-        auto from_col = [&](void *v, const void *blk, int col) {
-            return cudaMemcpy2DAsync(v, ld * cb, (const char *)blk + col * cb, 2 * cb, cb, (size_t)P,
+        auto from_col = [&](void *v, int b, const void *blk, int64_t col) {
+            return cudaMemcpy2DAsync(v, ld * cb, (const char *)blk + col * cb, width[b] * cb, cb, (size_t)P,
                                      cudaMemcpyDeviceToDevice, st);
         };
-        const int SV2 = sv_of(H, 2);
         static const double invf[5] = {1.0, 1.0, 0.5, 1.0 / 6.0, 1.0 / 24.0};
         // step t of bank b: the exponential from arr(b, t, 0) to arr(b, t + 1, 0)
         auto step = [&](int b, int64_t t, bool rec, double eps_r, bool cost, double eps_c) -> rsg_status {
@@ -2444,7 +2447,7 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
                     ep.ai = tau;
                     e = eps_c;
                 }
-                CKS(apply(H, pw[j], pw[j + 1], SV2, e, dir, ep, st));
+                CKS(apply(H, pw[j], pw[j + 1], sv_of(H, width[b]), e, dir, ep, st));
             }
             return RSG_OK;
         };
@@ -2452,15 +2455,17 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
         {
             const int64_t c = nck - 1, k0 = c * K, L = std::min<int64_t>(k0 + K, nsteps) - k0;
             const int b = (int)(c % 2);
-            CK(to_col(arr(b, 0, 0), 0, vec(ck0 + c)));
+            width[b] = ld;
+            CK(to_col(b, arr(b, 0, 0), 0, vec(ck0 + c)));
             for (int64_t t = 0; t < L * m; t++) CKS(step(b, t, true, eps[k0 + t / m], false, 0.0));
         }
         for (int64_t c = nck - 1; c >= 0; c--) {
             const int64_t k0c = c * K, k1c = std::min<int64_t>(k0c + K, nsteps), Tc = (k1c - k0c) * m;
             const int bc = (int)(c % 2), br = 1 - bc;
             const int64_t k0r = (c - 1) * K, Tr = c >= 1 ? (int64_t)K * m : 0;
-            CK(to_col(arr(br, 0, 0), 1, chi));
-            if (c >= 1) CK(to_col(arr(br, 0, 0), 0, vec(ck0 + c - 1)));
+            width[br] = c >= 1 ? 2 : ld;
+            CK(to_col(br, arr(br, 0, 0), width[br] - 1, chi));
+            if (c >= 1) CK(to_col(br, arr(br, 0, 0), 0, vec(ck0 + c - 1)));
             const int64_t T = std::max(Tc, Tr);
             for (int64_t t = 0; t < T; t++) {
                 const bool rec = t < Tr, cost = t < Tc;
@@ -2471,14 +2476,15 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
                     const int64_t tc = (k - k0c) * m + l;   // the costate's exponential in its segment's bank
                     const void *bb[4], *aa[4];
                     for (int j = 0; j < 4; j++) {
-                        bb[j] = (const char *)arr(br, t, j) + cb;
+                        bb[j] = (const char *)arr(br, t, j) + (width[br] - 1) * cb;
                         aa[j] = arr(bc, tc, j);
                     }
-                    CK(launch_adjoint_grad<R>(bb, aa, P, 2, H->Xd.as<R>(), h3, tau, H->dots.as<double>(), nba,
+                    CK(launch_adjoint_grad<R>(bb, aa, P, (int)width[br], (int)width[bc], H->Xd.as<R>(), h3, tau,
+                                              H->dots.as<double>(), nba,
                                               counter, H->grad.as<double>() + k, st));
                 }
             }
-            CK(from_col(chi, arr(br, Tc, 0), 1));
+            CK(from_col(chi, br, arr(br, Tc, 0), width[br] - 1));
         }
     }
     for (int64_t c = merged ? -1 : nck - 1; c >= 0; c--) {
@@ -2509,7 +2515,7 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
                 const void *aa[4] = {a0, keep_powers ? pslot(k - k0, l, 1) : pslot(0, l, 1),
                                      keep_powers ? pslot(k - k0, l, 2) : pslot(0, l, 2),
                                      keep_powers ? pslot(k - k0, l, 3) : pslot(0, l, 3)};
-                CK(launch_adjoint_grad<R>(bb, aa, P, (int)ld, H->Xd.as<R>(), h3, tau, H->dots.as<double>(), nba,
+                CK(launch_adjoint_grad<R>(bb, aa, P, (int)ld, (int)ld, H->Xd.as<R>(), h3, tau, H->dots.as<double>(), nba,
                                           counter, H->grad.as<double>() + k, st));
                 std::swap(chi, chi2);
             }

@@ -234,9 +234,10 @@ cudaError_t launch_adjoint_dots(const void *const *b, const void *const *a, int6
                                 const R *X, double h3, double *partial, int nblk,
                                 double *out, cudaStream_t st);
 // Fused adjoint inner products + reduction + grad_k update (one launch);
-// counter (device, zero on entry) is reset by the kernel.
+// counter (device, zero on entry) is reset by the kernel.  ldb, lda: row
+// lengths of the b and the a blocks.
 template <typename R>
-cudaError_t launch_adjoint_grad(const void *const *b, const void *const *a, int64_t P, int ld,
+cudaError_t launch_adjoint_grad(const void *const *b, const void *const *a, int64_t P, int ldb, int lda,
                                 const R *X, double h3, double tau, double *partial, int nblk,
                                 unsigned *counter, double *grad_k, cudaStream_t st);
 int adjoint_blocks(int64_t P);   // nblk of launch_adjoint_grad

@@ -391,8 +391,8 @@ __global__ void __launch_bounds__(256) k_adjoint_dots(const R *b0, const R *b1, 
 template <typename R>
 __global__ void __launch_bounds__(256) k_adjoint_grad(const R *b0, const R *b1, const R *b2, const R *b3,
                                                       const R *a0, const R *a1, const R *a2, const R *a3,
-                                                      int64_t P, int ld, const R *__restrict__ X, double h3,
-                                                      double tau, double *__restrict__ partial, int nblk,
+                                                      int64_t P, int ldb, int lda, const R *__restrict__ X,
+                                                      double h3, double tau, double *__restrict__ partial, int nblk,
                                                       unsigned *counter, double *grad_k) {
     // The gradient needs only sum_{i+j<=3} Im <b_j|X|a_i> / (i+j+1)!.  With
     // c_i = sum_{j<=3-i} b_j / (i+j+1)! (real weights) it is
@@ -407,11 +407,11 @@ __global__ void __launch_bounds__(256) k_adjoint_grad(const R *b0, const R *b1, 
     chain_begin();
     chain_wait();
     for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        const int64_t o = p * ld * 2;
+        const int64_t o = p * ldb * 2, q = p * lda * 2;
         const double br0 = widen(b0[o]), bi0 = widen(b0[o + 1]), br1 = widen(b1[o]), bi1 = widen(b1[o + 1]);
         const double br2 = widen(b2[o]), bi2 = widen(b2[o + 1]), br3 = widen(b3[o]), bi3 = widen(b3[o + 1]);
-        const double ar0 = widen(a0[o]), ai0 = widen(a0[o + 1]), ar1 = widen(a1[o]), ai1 = widen(a1[o + 1]);
-        const double ar2 = widen(a2[o]), ai2 = widen(a2[o + 1]), ar3 = widen(a3[o]), ai3 = widen(a3[o + 1]);
+        const double ar0 = widen(a0[q]), ai0 = widen(a0[q + 1]), ar1 = widen(a1[q]), ai1 = widen(a1[q + 1]);
+        const double ar2 = widen(a2[q]), ai2 = widen(a2[q + 1]), ar3 = widen(a3[q]), ai3 = widen(a3[q + 1]);
         // c_0 .. c_3
         const double c0r = fma(f4, br3, fma(f3, br2, fma(f2, br1, br0)));
         const double c0i = fma(f4, bi3, fma(f3, bi2, fma(f2, bi1, bi0)));
@@ -462,12 +462,12 @@ __global__ void __launch_bounds__(256) k_adjoint_grad(const R *b0, const R *b1, 
 int adjoint_blocks(int64_t P) { return (int)std::max<int64_t>(1, std::min<int64_t>(608, (P + 255) / 256)); }
 
 template <typename R>
-cudaError_t launch_adjoint_grad(const void *const *b, const void *const *a, int64_t P, int ld, const R *X,
-                                double h3, double tau, double *partial, int nblk, unsigned *counter,
+cudaError_t launch_adjoint_grad(const void *const *b, const void *const *a, int64_t P, int ldb, int lda,
+                                const R *X, double h3, double tau, double *partial, int nblk, unsigned *counter,
                                 double *grad_k, cudaStream_t st) {
     return launch_chained(k_adjoint_grad<R>, dim3(nblk), dim3(256), 0, st, true, (const R *)b[0], (const R *)b[1],
                           (const R *)b[2], (const R *)b[3], (const R *)a[0], (const R *)a[1], (const R *)a[2],
-                          (const R *)a[3], P, ld, X, h3, tau, partial, nblk, counter, grad_k);
+                          (const R *)a[3], P, ldb, lda, X, h3, tau, partial, nblk, counter, grad_k);
 }
 
 // Expand the 10 packed values into out[j*4+i] (complex double), zero elsewhere.
@@ -622,7 +622,8 @@ cudaError_t launch_grad_accum(const double *M, double tau, double *grad_k, cudaS
                                                 int, const R *, double, double *, int, double *,     \
                                                 cudaStream_t);                                       \
     template cudaError_t launch_adjoint_grad<R>(const void *const *, const void *const *, int64_t, int, \
-                                                const R *, double, double, double *, int, unsigned *,  \
+                                                int, const R *, double, double, double *, int,         \
+                                                unsigned *,                                            \
                                                 double *, cudaStream_t);                               \
     template cudaError_t launch_overlap<R>(const void *, const void *, int64_t, int, double,         \
                                            double *, int, double *, cudaStream_t);                   \
