@@ -81,11 +81,11 @@ def peaks():
 
 # stencil kernel of each "kernel" option value (rsg_ham_get_option "last_kernel")
 KERNEL_NAMES = {0: "k_apply_staged", 1: "k_apply_naive", 2: "k_apply_zmarch", 3: "k_apply_tma",
-                4: "k_apply_rowtma", 5: "k_apply_quad", 7: "k_apply_wide"}
+                4: "k_apply_rowtma", 5: "k_apply_quad", 7: "k_apply_wide"}   # 1 in complex128: k_apply_sum64 or k_apply_row64
 # the files the dominant stencil kernel (k_apply_wide) is compiled from; the
 # public header it also includes holds only C declarations the kernel does
 # not use
-KERNEL_SOURCES = ("rsg_wide.cu", "rsg_vec.cuh", "rsg_async.cuh", "rsg_internal.h")
+KERNEL_SOURCES = ("rsg_wide.cu", "rsg_vec.cuh", "rsg_async.cuh", "rsg_chain.cuh", "rsg_internal.h")
 
 
 def traffic_record(kernel_src_hash, kernel_name):

@@ -441,8 +441,12 @@ rsg_status rsg_batch_destroy(rsg_batch b);
  * (staged kernel: 16-byte vectors per point per block, 1, 2, 4 or 8),
  * "threads" (staged kernels: 256 or 512 threads per block; kernel 5: 256
  * gives 16 x 16 tiles, any other value 16 x 12 tiles with 192 threads).
- * Defaults: complex64 runs kernel 5 with 192 threads, 3 stages and 150-plane
- * z segments, complex128 kernel 1; kernels 0, 3 and 4 default to 256
+ * Defaults: complex64 runs kernel 7, 5 or 1 with a z segment length, by size
+ * (the kernel and segments whose blocks fill the SMs best; kernel 7 with whole
+ * columns on large blocks; the eigensolver and the shifted solves keep kernel
+ * 7, or 5 for narrow blocks, 1 when there are few tiles); complex128 kernel 1,
+ * with integer neighbour sums except on the smallest problems;
+ * kernels 0, 3 and 4 default to 256
  * threads, cv 2; 160 threads give kernel 5 16 x 10 tiles, three blocks per
  * SM (z segments up to 96 planes keep the three in shared memory).
  * "stages" (staged kernels: shared-memory pipeline depth, 3 or 4 for

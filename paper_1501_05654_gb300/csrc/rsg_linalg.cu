@@ -476,7 +476,8 @@ __global__ void __launch_bounds__(256) k_adjoint_grad(const R *b0, const R *b1, 
 }
 
 // Four blocks per SM: 28 FP64 instructions a point (two a clock per SM) need
-// every SM; one block per 2048 points left 24 of them idle at 64^3.
+// every SM; one block per 2048 points left 24 of them idle at 64^3 (28 and
+// 33 us, complex128 and complex64; now 24 to 25).
 int adjoint_blocks(int64_t P) { return (int)std::max<int64_t>(1, std::min<int64_t>(608, (P + 255) / 256)); }
 
 template <typename R>
