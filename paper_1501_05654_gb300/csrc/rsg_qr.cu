@@ -122,8 +122,9 @@ __global__ void __launch_bounds__(256) k_norms32(const float4 *__restrict__ psi,
 // ------------------------------------------------------- sums over blocks
 // out[i] = scale * sum_b partial[b][i], b in order: 32 outputs per block,
 // whose rows are staged 32 at a time by 1024 threads while one warp adds them
-// (the additions are the chain that bounds it, about 12 us for 608 rows; with
-// the loads in that chain too it took 100 us).
+// (the additions are the chain that bounds it, 29 us for 608 rows whether one
+// or four groups of loads are in flight; with the loads in that chain too it
+// took 100 us).
 __global__ void __launch_bounds__(1024) k_sum_rows(const double *__restrict__ partial, int nblk, int64_t n,
                                                    double scale, double *__restrict__ out) {
     __shared__ double buf[2][32][33];
