@@ -518,9 +518,10 @@ __device__ void bs_dot(const SysArgs &S, int atom, int src, unsigned char *sm) {
     double *red = (double *)sm;
     double *cv = red + NP * 4 * kBNT;
     int *qs = (int *)(cv + NP * 4 * kBMaxLd / 2);
-    const int q0 = __ldg(S.chunk_q0 + __ldg(S.atom_chunk0 + atom));
-    const int q1 = __ldg(S.chunk_q1 + __ldg(S.atom_chunk0 + atom + 1) - 1);
-    const int nq = q1 - q0;
+    // an atom whose sphere holds no mesh point has no chunk: no entries, D = 0
+    const int c0 = __ldg(S.atom_chunk0 + atom), c1 = __ldg(S.atom_chunk0 + atom + 1);
+    const int q0 = c0 < c1 ? __ldg(S.chunk_q0 + c0) : 0;
+    const int nq = c0 < c1 ? __ldg(S.chunk_q1 + c1 - 1) - q0 : 0;
     const bool staged = (size_t)((unsigned char *)(qs + nq) - sm) <= (size_t)kBNS * kBSlot;
     if (staged) {
 #pragma unroll 4
