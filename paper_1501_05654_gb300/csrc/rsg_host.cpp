@@ -139,8 +139,17 @@ struct DevBuf {
     cudaError_t upload(const std::vector<T> &v) {
         cudaError_t e = ensure(v.size() * sizeof(T));
         if (e != cudaSuccess || v.empty()) return e;
-        return cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+        return e != cudaSuccess ? e : landed();
     }
+    cudaError_t zero(size_t bytes) {
+        cudaError_t e = cudaMemset(p, 0, bytes);
+        return e != cudaSuccess ? e : landed();
+    }
+    // A copy from pageable memory may return before its last piece is on the
+    // device, and a memset always may; a kernel on a non-blocking stream does
+    // not wait for the legacy stream.
+    static cudaError_t landed() { return cudaStreamSynchronize(cudaStreamLegacy); }
     template <typename T>
     T *as() const {
         return (T *)p;
@@ -2996,10 +3005,10 @@ rsg_status batch_build_step(rsg_batch b) {
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     b->nblocks = std::max(1, std::min(sms, (int)b->stage_items.size()));
     CK(b->d_status.ensure(sizeof(int)));
-    CK(cudaMemset(b->d_status.p, 0, sizeof(int)));
+    CK(b->d_status.zero(sizeof(int)));
     CK(b->d_ctl.ensure(sizeof(BCtl)));
     CK(b->d_zero.ensure(kBZeroBytes));
-    CK(cudaMemset(b->d_zero.p, 0, kBZeroBytes));
+    CK(b->d_zero.zero(kBZeroBytes));
     b->step_nst = 0;   // items and counters follow the scheme at capture
     b->batched = true;
     b->n_launch_step = 1;
@@ -3163,7 +3172,7 @@ rsg_status rsg_batch_propagate(rsg_batch b, void *const *psis, int64_t nsteps, d
         CK(cudaMemcpyAsync(&s, b->d_status.p, sizeof(int), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         if (s != 0) {
-            CK(cudaMemset(b->d_status.p, 0, sizeof(int)));
+            CK(b->d_status.zero(sizeof(int)));
             return fail(RSG_ERR_TIMEOUT, "a bounded wait of the batched step gave up");
         }
     }
