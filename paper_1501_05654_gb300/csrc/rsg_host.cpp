@@ -978,7 +978,7 @@ rsg_status orthonormalize_dev(rsg_ham H, void *psi, int64_t S, int64_t ld, doubl
         CK(cudaMemsetAsync(H->status.p, 0, sizeof(int), st));
     }
     if (H->dtype == RSG_C64) {
-        // FP64 norms for the diagonal, FP32 runs summed in FP64 elsewhere
+        // FP64 norms for the diagonal, FP32 runs in two-float and FP64 sums elsewhere
         const size_t nrm_bytes = ((size_t)S * sizeof(double) + 255) / 256 * 256;
         CK(H->Wc.ensure(nrm_bytes + tri_c64_bytes((int)S)));
         double *nrm = H->Wc.as<double>();

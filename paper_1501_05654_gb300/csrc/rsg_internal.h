@@ -202,8 +202,9 @@ template <typename R>
 cudaError_t launch_gram(const void *psi, int64_t P, int ld, int S, double h3,
                         double *partial, int nblk, double *G, cudaStream_t st);
 int gram_blocks(int64_t P, int S);
-// complex64 Gram: FP32 products in runs of 8 points, runs summed in FP64;
-// the diagonal is replaced by the given FP64 norms (h3 applied).
+// complex64 Gram: FP32 products in runs of 8 points, up to 128 runs in a
+// two-float sum, those summed in FP64; the diagonal is replaced by the given
+// FP64 norms (h3 applied).
 cudaError_t launch_gram_c64(const void *psi, int64_t P, int ld, int S, double h3, double *partial,
                             int nblk, double *G, const double *norms, cudaStream_t st);
 // complex64 triangular update with W^H rounded to FP32 (Wt_buf: tri_c64_bytes(S)

@@ -138,16 +138,11 @@ __global__ void __launch_bounds__(256) k_resid(const R *__restrict__ x, const R 
     if (threadIdx.x == 0) partial[(int64_t)blockIdx.x * S + s] = red[0];
 }
 
-// FP32 <-> FP64 in integer arithmetic.  A conversion instruction takes two
+// FP64 to FP32 in integer arithmetic (FP32 to FP64: widen, rsg_vec.cuh).  A conversion instruction takes two
 // slots of the FP64 pipe (two a clock per SM), which bounds the complex64
 // vector updates below; exponents that need denormal or special handling take
 // the instruction.  R = 14 sphere x 8 states: update 293 to 91 us (with the
 // unit scale of x dropped and 16-byte accesses), bilinear form 251 to 139 us.
-__device__ __forceinline__ double widen(float f) {
-    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
-    if (e == 0u || e == 0x7f800000u) return (u & 0x7fffffffu) == 0u ? __hiloint2double((int)u, 0) : (double)f;
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
-}
 __device__ __forceinline__ double widen(double d) { return d; }
 // one complex value (8- or 16-byte aligned) in one load: the adjoint's
 // gradient kernel waits for loads (9 a point instead of 17; 64^3 complex128 25.0

@@ -7,9 +7,10 @@
 // 0.23 T FP32 FMAs on a 7.25 GB block, so FP32 arithmetic (about 7 ms each at
 // the SIMT rate) and not memory (1.1 ms a pass) is the floor.  Both are
 // register-tiled products.  FP64 instructions (two a clock per SM) are kept
-// off the inner loops: runs of FP32 sums are collected in two-float sums (48
-// bits) and meet FP64 once per block.
+// off the inner loops: runs of FP32 sums are collected in short two-float sums
+// before they meet FP64.
 #include <algorithm>
+#include <type_traits>
 
 #include "rsg_async.cuh"
 #include "rsg_internal.h"
@@ -187,14 +188,19 @@ __global__ void __launch_bounds__(256) k_sum_herm(const double2 *__restrict__ pa
 // Tile TS x TS of (s, t), tiles with s-tile <= t-tile; a thread owns 4 x 4
 // entries and TS^2 / 16 threads make a group.  Below 64 columns the 256
 // threads are several groups that share the staged points.  FP32 products
-// are summed in FP32 over runs of 8 points; each run is collected in a
-// two-float sum, converted to FP64 at the end of the block's points.  The
-// points come as they lie (one 16-byte asynchronous copy per two states),
-// double-buffered; on the diagonal both operands are the same panel.
-// 192^3 x 128 states: 17.1 ms (108 ms when every run met two FP64 additions
-// and conversions per value; 27.9 with panels rearranged through registers).
+// are summed in FP32 over runs of 8 points; kGHeld runs are collected in a
+// two-float sum (whose own rounding, below 2^-37 of its largest partial sum,
+// lies under the 2^-24 of the runs), which is added to an FP64 sum.  A block
+// in which such a sum leaves the FP32 range although its runs do not (squares
+// near 1e36) sums its points again, every run in FP64.  The points come as
+// they lie (one 16-byte asynchronous copy per two states), double-buffered;
+// on the diagonal both operands are the same panel.  192^3 x 128 states: 19
+// ms (108 ms when every run met two FP64 additions and conversions per value;
+// kGHeld = 64 adds 0.6 ms, one two-float sum for all of a block's points, of
+// less range and fewer bits, saves 2; FP64 sums in shared memory save nothing).
 // The point blocks are `nsub` pieces of the blocks of 4096 points or more
 // that gram_blocks names, cut at multiples of a run.
+constexpr int kGHeld = 128;   // runs in a two-float sum
 template <int TS>
 struct G32Shape {
     static constexpr int NTH = TS * TS / 16, NG = 256 / NTH, RUNS = TS == 64 ? 4 : 2, KP = 8 * RUNS * NG;
@@ -252,54 +258,89 @@ __global__ void __launch_bounds__(256, 1) k_gram32(const float2 *__restrict__ ps
         }
         cp_async_commit();
     };
-    // two-float sums of the 4 x 4 entries: (re, im) pairs
-    float2 hi[4][4], lo[4][4];
+    double2 tot[4][4];   // sums of the 4 x 4 entries
+    // PLAIN: every run added in FP64 by itself
+    auto sum_points = [&](auto plain) {
+        constexpr bool PLAIN = decltype(plain)::value;
+        float2 hi[4][4], lo[4][4];   // two-float sums of up to kGHeld runs, (re, im) pairs
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+        for (int i = 0; i < 4; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) hi[i][j] = lo[i][j] = make_float2(0.f, 0.f);
-    if (p0 < p1) stage(p0, 0);
-    int k = 0;
-    for (int64_t pc = p0; pc < p1; pc += KP, k ^= 1) {
-        cp_async_wait<0>();
-        __syncthreads();
-        if (pc + KP < p1) stage(pc + KP, k ^ 1);
-        if (skip) continue;
-        const float2 *A = buf + k * BUFST + sr, *B = buf + k * BUFST + (TS == 64 && !diag ? G::PANEL : 0) + tc;
-#pragma unroll 1
-        for (int h = 0; h < G::RUNS; h++) {
-            float2 f[4][4];
+            for (int j = 0; j < 4; j++) {
+                hi[i][j] = lo[i][j] = make_float2(0.f, 0.f);
+                tot[i][j] = make_double2(0.0, 0.0);
+            }
+        auto flush = [&]() {
 #pragma unroll
             for (int i = 0; i < 4; i++)
 #pragma unroll
-                for (int j = 0; j < 4; j++) f[i][j] = make_float2(0.f, 0.f);
+                for (int j = 0; j < 4; j++) {
+                    tot[i][j].x += widen(hi[i][j].x) + widen(lo[i][j].x);
+                    tot[i][j].y += widen(hi[i][j].y) + widen(lo[i][j].y);
+                    hi[i][j] = lo[i][j] = make_float2(0.f, 0.f);
+                }
+        };
+        if (p0 < p1) stage(p0, 0);
+        int k = 0, held = 0;
+#pragma unroll 1
+        for (int64_t pc = p0; pc < p1; pc += KP, k ^= 1) {
+            cp_async_wait<0>();
+            __syncthreads();
+            if (pc + KP < p1) stage(pc + KP, k ^ 1);
+            if (skip) continue;
+            const float2 *A = buf + k * BUFST + sr, *B = buf + k * BUFST + (TS == 64 && !diag ? G::PANEL : 0) + tc;
+#pragma unroll 1
+            for (int h = 0; h < G::RUNS; h++) {
+                float2 f[4][4];
 #pragma unroll
-            for (int q = 0; q < 8; q++) {
-                const int row = ((g * G::RUNS + h) * 8 + q) * TS;
-                const float4 a0 = *(const float4 *)(A + row), a1 = *(const float4 *)(A + row + 8);
-                const float4 b0v = *(const float4 *)(B + row), b1v = *(const float4 *)(B + row + 2 * LX);
-                const float2 x[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
-                                     make_float2(a1.z, a1.w)};
-                const float2 y[4] = {make_float2(b0v.x, b0v.y), make_float2(b0v.z, b0v.w), make_float2(b1v.x, b1v.y),
-                                     make_float2(b1v.z, b1v.w)};
+                for (int i = 0; i < 4; i++)
+#pragma unroll
+                    for (int j = 0; j < 4; j++) f[i][j] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int q = 0; q < 8; q++) {
+                    const int row = ((g * G::RUNS + h) * 8 + q) * TS;
+                    const float4 a0 = *(const float4 *)(A + row), a1 = *(const float4 *)(A + row + 8);
+                    const float4 b0v = *(const float4 *)(B + row), b1v = *(const float4 *)(B + row + 2 * LX);
+                    const float2 x[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
+                                         make_float2(a1.z, a1.w)};
+                    const float2 y[4] = {make_float2(b0v.x, b0v.y), make_float2(b0v.z, b0v.w),
+                                         make_float2(b1v.x, b1v.y), make_float2(b1v.z, b1v.w)};
+#pragma unroll
+                    for (int i = 0; i < 4; i++)
+#pragma unroll
+                        for (int j = 0; j < 4; j++) {
+                            // conj(x) y
+                            f[i][j].x = fmaf(x[i].x, y[j].x, fmaf(x[i].y, y[j].y, f[i][j].x));
+                            f[i][j].y = fmaf(x[i].x, y[j].y, fmaf(-x[i].y, y[j].x, f[i][j].y));
+                        }
+                }
 #pragma unroll
                 for (int i = 0; i < 4; i++)
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
-                        // conj(x) y
-                        f[i][j].x = fmaf(x[i].x, y[j].x, fmaf(x[i].y, y[j].y, f[i][j].x));
-                        f[i][j].y = fmaf(x[i].x, y[j].y, fmaf(-x[i].y, y[j].x, f[i][j].y));
+                        if constexpr (PLAIN) {
+                            tot[i][j].x += (double)f[i][j].x;
+                            tot[i][j].y += (double)f[i][j].y;
+                        } else {
+                            f2_two_sum(hi[i][j], lo[i][j], f[i][j]);
+                        }
                     }
             }
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) f2_two_sum(hi[i][j], lo[i][j], f[i][j]);
+            if (!PLAIN && (held += G::RUNS) >= kGHeld) {
+                flush();
+                held = 0;
+            }
         }
-    }
-    auto val = [&](int i, int j) {
-        return make_double2((double)hi[i][j].x + (double)lo[i][j].x, (double)hi[i][j].y + (double)lo[i][j].y);
+        if (!PLAIN && !skip) flush();
     };
+    sum_points(std::false_type{});
+    // runs that FP32 holds while their two-float sum does not
+    bool over = false;
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) over = over || !isfinite(tot[i][j].x) || !isfinite(tot[i][j].y);
+    if (__syncthreads_or(over)) sum_points(std::true_type{});
     auto row_of = [&](int i) { return sr + (i & 1) + 8 * (i >> 1); };
     auto col_of = [&](int j) { return tc + (j & 1) + 2 * LX * (j >> 1); };
     if constexpr (G::NG == 1) {
@@ -309,7 +350,7 @@ __global__ void __launch_bounds__(256, 1) k_gram32(const float2 *__restrict__ ps
 #pragma unroll
             for (int j = 0; j < 4; j++) {
                 const int s = s0 + row_of(i), t = t0 + col_of(j);
-                if (s < S && t < S) partial[((int64_t)blockIdx.z * S + s) * S + t] = val(i, j);
+                if (s < S && t < S) partial[((int64_t)blockIdx.z * S + s) * S + t] = tot[i][j];
             }
     } else {
         __syncthreads();
@@ -317,7 +358,7 @@ __global__ void __launch_bounds__(256, 1) k_gram32(const float2 *__restrict__ ps
 #pragma unroll
         for (int i = 0; i < 4; i++)
 #pragma unroll
-            for (int j = 0; j < 4; j++) red[(g * TS + row_of(i)) * TS + col_of(j)] = val(i, j);
+            for (int j = 0; j < 4; j++) red[(g * TS + row_of(i)) * TS + col_of(j)] = tot[i][j];
         __syncthreads();
         for (int e = tid; e < TS * TS; e += 256) {
             const int s = s0 + e / TS, t = t0 + e % TS;

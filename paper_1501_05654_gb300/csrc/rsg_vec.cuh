@@ -42,6 +42,15 @@ __device__ __forceinline__ float2 f2_mul(float2 a, float2 b) {
     return d.f;
 }
 
+// FP32 to FP64 in integer arithmetic: a conversion instruction takes two slots
+// of the FP64 pipe (two a clock per SM).  Exponents that need denormal or
+// special handling take the instruction.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return (u & 0x7fffffffu) == 0u ? __hiloint2double((int)u, 0) : (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
 template <>
 struct VT<float> {
     using T = float4;
