@@ -24,32 +24,39 @@ __device__ __forceinline__ float2 f2_neg(float2 a) { return make_float2(-a.x, -a
 // a - b (exact product, so one rounding)
 __device__ __forceinline__ float2 f2_sub(float2 a, float2 b) { return f2_fma(b, make_float2(-1.f, -1.f), a); }
 
-// (hi, lo) += r: hi takes the rounded sum, lo the exact rounding error of it
-// (Knuth's two-sum), per component
-__device__ __forceinline__ void f2_two_sum(float2 &hi, float2 &lo, float2 r) {
+// hi += r, rounded; returns the exact rounding error (Knuth's two-sum), per
+// component
+__device__ __forceinline__ float2 f2_add_err(float2 &hi, float2 r) {
     const float2 s = f2_add(hi, r);
     const float2 b = f2_sub(s, hi);
     const float2 e = f2_add(f2_sub(hi, f2_sub(s, b)), f2_sub(r, b));
     hi = s;
+    return e;
+}
+// (hi, lo) += r: hi takes the rounded sum, lo the rounding error of it
+__device__ __forceinline__ void f2_two_sum(float2 &hi, float2 &lo, float2 r) {
+    const float2 e = f2_add_err(hi, r);
     lo = f2_add(lo, e);
 }
 
 // ------------------------------------------------------------------ norms
 // partial[blk][s] = sum over the block's points of |psi[p,s]|^2.  A thread
 // owns a 16-byte vector (two states) of every by-th point.  The squares of
-// four points are summed as an exact two-float sum (each square split by an
-// FMA into its rounded value and its error) and added to FP64 once: half an
-// FP64 instruction per value instead of four, which makes the pass
-// memory-bound.  A group whose sum leaves the range where FP32 squares and
-// their errors are exact (tails, huge values) is summed again in FP64.
-// 192^3 x 128 states: 1.78 ms (8.6 ms when every square was an FP64 FMA).
-constexpr int kNRun = 4;
+// eight points (each split by an FMA into its rounded value and its error) are
+// summed in three floats: the second takes the exact rounding errors of the
+// first, the third those of the second, so that less than 2^-60 of the sum is
+// lost before it is added to FP64 once.  A group whose sum leaves the range
+// where FP32 squares and their errors are exact (tails, huge values) is summed
+// again in FP64.  Relative error of the norms, rms: 1e-16 to 2.5e-16 (every
+// square an FP64 FMA: 1e-16 to 1e-15; two floats: 7e-16).  Bound by the issue of
+// the packed additions: 192^3 x 128 states 1.85 ms (8.6 ms with FP64 FMAs).
+constexpr int kNRun = 8;
 constexpr float kNLow = 1e-24f, kNHigh = 1e37f;
-// Adds state c's part of a group, of which at least one state is outside the
-// exact range.
-__device__ __forceinline__ void add_outside(const float4 (&x)[kNRun], float hi, float lo, int c, double &a) {
+// Adds state c's part of a group: its three-float sum, or its squares in FP64
+// outside the exact range.
+__device__ __forceinline__ void add_group(const float4 (&x)[kNRun], float hi, float lo, float l2, int c, double &a) {
     if (hi >= kNLow && hi <= kNHigh) {
-        a += (double)hi + (double)lo;
+        a += widen(hi) + (widen(lo) + widen(l2));
         return;
     }
     bool zero = true;
@@ -82,7 +89,7 @@ __global__ void __launch_bounds__(256) k_norms32(const float4 *__restrict__ psi,
                     x[k] = q < p1 ? __ldg(psi + q * ldv + v) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
                 // components (state 0, state 1): re then im of each point
-                float2 hi = make_float2(0.f, 0.f), lo = hi;
+                float2 hi = make_float2(0.f, 0.f), lo = hi, l2 = hi;
 #pragma unroll
                 for (int k = 0; k < kNRun; k++) {
 #pragma unroll
@@ -90,17 +97,13 @@ __global__ void __launch_bounds__(256) k_norms32(const float4 *__restrict__ psi,
                         const float2 u = c ? make_float2(x[k].y, x[k].w) : make_float2(x[k].x, x[k].z);
                         const float2 sq = f2_mul(u, u);
                         const float2 er = f2_fma(u, u, f2_neg(sq));
-                        f2_two_sum(hi, lo, sq);
-                        lo = f2_add(lo, er);
+                        const float2 e = f2_add_err(hi, sq);
+                        f2_two_sum(lo, l2, e);
+                        f2_two_sum(lo, l2, er);
                     }
                 }
-                if (hi.x >= kNLow && hi.x <= kNHigh && hi.y >= kNLow && hi.y <= kNHigh) {
-                    a0 += (double)hi.x + (double)lo.x;
-                    a1 += (double)hi.y + (double)lo.y;
-                } else {
-                    add_outside(x, hi.x, lo.x, 0, a0);
-                    add_outside(x, hi.y, lo.y, 1, a1);
-                }
+                add_group(x, hi.x, lo.x, l2.x, 0, a0);
+                add_group(x, hi.y, lo.y, l2.y, 1, a1);
             }
         }
         const int tid = threadIdx.y * bx + threadIdx.x;
