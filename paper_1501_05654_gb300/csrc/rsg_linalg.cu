@@ -92,12 +92,43 @@ __global__ void __launch_bounds__(kRowsNT) k_rows(R *psi, int64_t P, int ld, int
     }
 }
 
+// The same for blocks so wide that a row and a row of M do not fit in shared
+// memory together (above 7,264 states): one point per block, M from global
+// memory.
+template <typename R, bool TRI>
+__global__ void __launch_bounds__(kRowsNT) k_rows_wide(R *psi, int ld, int S, const double2 *__restrict__ M) {
+    extern __shared__ double2 rsm[];
+    R *row = psi + (int64_t)blockIdx.x * ld * 2;
+    for (int t = threadIdx.x; t < S; t += kRowsNT) ld_c(row + 2 * t, rsm[t].x, rsm[t].y);
+    __syncthreads();
+    for (int s = threadIdx.x; s < S; s += kRowsNT) {
+        double re = 0.0, im = 0.0;
+        const int te = TRI ? s + 1 : S;
+        for (int t = 0; t < te; t++) {
+            const double2 a = rsm[t];
+            double2 m = M[TRI ? (int64_t)s * S + t : (int64_t)t * S + s];
+            if (TRI) m.y = -m.y;
+            re = fma(a.x, m.x, fma(-a.y, m.y, re));
+            im = fma(a.x, m.y, fma(a.y, m.x, im));
+        }
+        row[2 * s] = (R)re;
+        row[2 * s + 1] = (R)im;
+    }
+}
+
 template <typename R, bool TRI>
 cudaError_t rows_launch(void *psi, int64_t P, int ld, int S, const double *M, cudaStream_t st) {
     // one item per thread, fewer points where the rows would not fit
     const int ng = (S + 3) / 4, pt = std::max(1, kRowsNT / ng), nt = std::min(S, std::max(1, kRowsChunk / S));
     const size_t smem = ((size_t)pt * S + (size_t)nt * S) * sizeof(double2);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
+    if (smem > 227 * 1024) {
+        const size_t row = (size_t)S * sizeof(double2);
+        if (row > 227 * 1024) return cudaErrorInvalidValue;
+        cudaError_t e = cudaFuncSetAttribute(k_rows_wide<R, TRI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row);
+        if (e != cudaSuccess) return e;
+        k_rows_wide<R, TRI><<<(unsigned)P, kRowsNT, row, st>>>((R *)psi, ld, S, (const double2 *)M);
+        return cudaGetLastError();
+    }
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_rows<R, TRI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
