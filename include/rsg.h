@@ -462,7 +462,10 @@ rsg_status rsg_batch_destroy(rsg_batch b);
  * memory, the default), "proj_overlap" (1: the projector
  * coefficients of each application run on an internal side stream next to
  * the stencil, which does not read them, and the projector terms after the
- * stencil wait for them; 0, the default: all on the caller's stream).
+ * stencil wait for them; 0, the default: all on the caller's stream),
+ * "sum_planes" (complex128 kernel 1: planes per block of the integer
+ * neighbour sums, 1..32, 0 for FP64 sums, -1 by size, the default; image walls
+ * and complex scaling always add in FP64).
  * A shape whose shared memory does not fit the SM fails with RSG_ERR_CUDA. */
 rsg_status rsg_ham_set_option(rsg_ham H, const char *key, int64_t value);
 
@@ -479,7 +482,10 @@ rsg_status rsg_ham_autotune(rsg_ham H, const void *psi, void *work, int64_t S, i
 /* Reads an option set above, or "last_kernel": the stencil kernel (0..5, or
  * 6 for the complex-scaled operator)
  * that the last Hamiltonian application actually ran (-1 before any), after
- * automatic fallbacks (small problems, TMA unavailable). */
+ * automatic fallbacks (small problems, TMA unavailable); "last_zseg": its
+ * planes per z segment (0 for kernels 1 and 6, which have none);
+ * "last_sum_planes": its planes per block with integer neighbour sums (0: FP64
+ * or complex64 sums). */
 rsg_status rsg_ham_get_option(rsg_ham H, const char *key, int64_t *value);
 
 /* Measurement hooks.  rsg_ham_profile(H, 1) starts recording a CUDA event

@@ -190,6 +190,9 @@ struct rsg_ham_s {
     // the sums and planes per block of kernel 1, per vectors per point
     std::map<std::tuple<int, bool, bool>, TileCfg> auto_cfg;
     int last_kernel = -1;        // stencil kernel of the last application
+    int last_zseg = 0;           // its planes per z segment (tiled kernels)
+    int last_sum = 0;            // its planes per block with integer neighbour sums (complex128), 0: FP64 sums
+    int sum_planes = -1;         // option "sum_planes": 0..32 as last_sum, -1 by size
     int adj_keep = -1;           // adjoint: keep segment powers (1), recompute (0), by memory (-1)
     int adj_merge = -1;          // adjoint: costate and recompute sweeps share launches (1), not (0), auto (-1)
     // projectors
@@ -779,7 +782,9 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
     // two-column applications run on the one-thread-per-value kernel
     if (ep.twocol) cfg.kernel = 1;
     if (H->dtype == RSG_C128 && cfg.kernel == 1 && m->bc == RSG_BC_ZERO && !H->has_scaling)
-        cfg.sum_zs = choose_c128(H, SV);
+        cfg.sum_zs = H->sum_planes >= 0 ? H->sum_planes : choose_c128(H, SV);
+    H->last_zseg = 0;
+    H->last_sum = cfg.sum_zs;
     if (cfg.kernel != 1) {
         int TX, TY;
         block_shape(cfg, SV, &TX, &TY);
@@ -903,6 +908,7 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
         CK(launch_proj_scatter<R>(a, H->pj, st));
         H->n_launch++;
     }
+    if (H->last_kernel != 1 && H->last_kernel != 6) H->last_zseg = cfg.zseg;
     // algorithmic bytes: read u, write out, optional base / acc (read+write),
     // the potential, and (with projectors) the per-point entry lists,
     // entry values and the coefficient block
@@ -1283,6 +1289,9 @@ rsg_status rsg_ham_get_option(rsg_ham H, const char *key, int64_t *value) {
     std::string k(key);
     if (k == "kernel") *value = H->cfg.kernel;
     else if (k == "last_kernel") *value = H->last_kernel;
+    else if (k == "last_zseg") *value = H->last_zseg;
+    else if (k == "last_sum_planes") *value = H->last_sum;
+    else if (k == "sum_planes") *value = H->sum_planes;
     else if (k == "rx") *value = H->cfg.rx;
     else if (k == "ty") *value = H->cfg.ty;
     else if (k == "wide_ty") *value = H->cfg.wty;
@@ -1315,6 +1324,7 @@ rsg_status rsg_ham_set_option(rsg_ham H, const char *key, int64_t value) {
     else if (k == "adjoint_keep_powers" && value >= -1 && value <= 1) H->adj_keep = (int)value;
     else if (k == "adjoint_merge" && value >= -1 && value <= 1) H->adj_merge = (int)value;
     else if (k == "proj_overlap" && (value == 0 || value == 1)) H->proj_overlap = (int)value;
+    else if (k == "sum_planes" && value >= -1 && value <= 32) H->sum_planes = (int)value;
     else if (k == "threads" && (value == 160 || value == 192 || value == 256 || value == 512))
         H->cfg.threads = (int)value;
     else if (k == "sync" && value >= 0 && value <= 2) H->cfg.sync = (int)value;
