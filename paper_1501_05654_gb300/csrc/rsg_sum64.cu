@@ -10,25 +10,32 @@
 // arithmetic.  The FP64 pipe does two instructions a clock per SM, and 40 of
 // the 56 a value needs are the additions of the six neighbours at one
 // distance.  Here the six values of a shell are added as 64-bit integers:
-// each double is split once into a signed mantissa (53 bits, seven guard bits
-// below) and an exponent, the mantissas are shifted to the largest exponent
-// of the six, and the sum is rounded once when it is converted back.  A
-// value cut off by the shift loses less than 2^-60 of the largest of the six,
-// so a shell sum is at least as exact as five FP64 additions, whatever the
-// range of the values; the weights, the diagonal and the epilogue stay FP64.
-// Sums that hold Inf or NaN, or lie at the ends of the exponent range, take a
-// slow path.
+// each double is split once into a mantissa (53 bits, seven guard bits below)
+// and an exponent, the mantissas are shifted to the largest exponent of the
+// six, and the sum is rounded once when it is converted back.  A value cut off
+// by the shift loses less than 2^-59 of the largest of the six, so a shell
+// sum is off by less than 5 x 2^-59 of the largest before its one rounding
+// (five FP64 additions round five times, by up to 2^-53 of their sums); where
+// the largest cancel, that is the bound on what is left.  Negative values are
+// kept as one's complements, which the arithmetic shift cuts off towards zero
+// like positive ones, and every sum adds one per negative value: the sum is
+// odd, H(-u) = -H(u) in every bit, and opposite values cancel.  The weights,
+// the diagonal and the epilogue stay FP64.  Sums that hold Inf or NaN, or lie
+// at the ends of the exponent range, take a slow path.
 //
 // A block owns a TX x TY tile of columns for NSC states and marches along z:
 // a thread keeps its column's nine split values, the plane's tile and halo
 // lie split in shared memory (two slots, one barrier a plane).  Bound by
 // instruction issue at 16 warps per SM (128 registers); the FP64 pipe is
-// about a third busy.  904,089 points (R = 12 sphere) x 16 states: 1.11 ms
-// (1.79 ms with FP64 sums, whose floor is 1.39 ms); 61^3 x 8: 0.129 ms (0.234);
-// 64^3 x 2 columns: 43.6 us (68).  Converting the sums with the conversion
-// instruction instead of integers costs 10% (two FP64 slots each).  Error
-// against 80-bit sums on noise, packets and values spread over 2^+-900, of
-// the norm: 1.35e-16, 9.8e-16, 1.1e-16 (FP64 sums 1.39e-16, 1.1e-15, 1.1e-16).
+// about a third busy.  Horner stages without projectors, in a chain of steps,
+// against FP64 sums: 904,089 points (R = 12 sphere) x 16 states 1.06 ms (1.65);
+// 61^3 x 8 0.121 (0.209); 96^3 x 3 0.168 (0.292); 64^3 x 2 columns 39.7 us (59.2);
+// 32^3 x 4 12.7 us (16.9).  Two's complements, whose shift cuts negative values
+// off downwards, would save 6%, and H(-u) would differ from -H(u) in places.
+// Converting the sums with the conversion instruction instead of integers costs
+// 10% (two FP64 slots each).  Error against 80-bit sums on noise, packets and
+// values spread over 2^+-900, of the norm: 1.35e-16, 9.8e-16, 1.1e-16 (FP64 sums
+// 1.39e-16, 1.1e-15, 1.1e-16).
 #include "rsg_async.cuh"
 #include "rsg_chain.cuh"
 #include "rsg_internal.h"
@@ -41,7 +48,7 @@ namespace {
 
 constexpr int kSumTX = 16, kSumNT = 256, kSumMaxZ = 32;
 struct SplitC {
-    long long re, im;
+    long long re, im;   // mantissas, one's complement
     int e;   // exponents, re in the low half
 };
 __device__ __forceinline__ long long split_real(double d, int &e) {
@@ -50,7 +57,7 @@ __device__ __forceinline__ long long split_real(double d, int &e) {
     const unsigned mh = ((unsigned)hi & 0xfffffu) | (eb ? 0x100000u : 0u);
     long long m = (long long)(((unsigned long long)mh << 32 | (unsigned)__double2loint(d)) << 7);
     e = eb ? (int)eb : 1;
-    return hi < 0 ? -m : m;
+    return m ^ (long long)(hi >> 31);
 }
 __device__ __forceinline__ SplitC split(const double2 &d) {
     SplitC s;
@@ -66,7 +73,7 @@ __device__ __noinline__ double shell_slow(long long S, int E, const long long *m
         double t = 0.0;
         for (int i = 0; i < 6; i++)
             if (e[i] == 0x7ff) {
-                const unsigned long long a = (unsigned long long)(m[i] < 0 ? -m[i] : m[i]) >> 7;
+                const unsigned long long a = (unsigned long long)(m[i] < 0 ? ~m[i] : m[i]) >> 7;
                 t += __hiloint2double((m[i] < 0 ? 0xfff00000 : 0x7ff00000) | (int)((a >> 32) & 0xfffff), (int)a);
             }
         return t;
@@ -218,13 +225,19 @@ __global__ void __launch_bounds__(kSumNT, 2) k_apply_sum64(const ApplyArgs<doubl
                 unsigned E = (unsigned)e[0];
 #pragma unroll
                 for (int j = 1; j < 6; j++) E = __vmaxu2(E, (unsigned)e[j]);
+                // the one's complements of the negative terms are one too low each
                 long long sr = 0, si = 0;
+                int nr = 0, ni = 0;
 #pragma unroll
                 for (int j = 0; j < 6; j++) {
                     const unsigned d = E - (unsigned)e[j];   // each half >= 0: no borrow
                     sr += shift_down(m[j].x, d & 0xffff);
                     si += shift_down(m[j].y, d >> 16);
+                    nr += (int)((unsigned long long)m[j].x >> 63);
+                    ni += (int)((unsigned long long)m[j].y >> 63);
                 }
+                sr += nr;
+                si += ni;
                 const int er = (int)(E & 0xffff), ei = (int)(E >> 16);
                 bool slr, sli;
                 double2 s = make_double2(shell_round(sr, er, slr), shell_round(si, ei, sli));
