@@ -22,6 +22,8 @@
  *   - All calls return an rsg_status; rsg_last_error() gives a thread-local
  *     message for the last failure.  No exception crosses the ABI.
  *   - Handles are owned by the library; destroy them with the matching call.
+ *     A Hamiltonian or batch is used by one host thread at a time; several
+ *     Hamiltonians on one mesh may be used by different threads at once.
  *     The caller owns every state, potential, field and gradient buffer.
  *   - State blocks are DEVICE pointers to a row-major (P, ld) array of
  *     complex values, states fastest: element (p, s) at offset p*ld + s.

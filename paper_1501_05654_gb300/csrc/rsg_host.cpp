@@ -27,6 +27,7 @@
 #include <unistd.h>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <type_traits>
@@ -169,6 +170,9 @@ struct rsg_mesh_s {
     std::vector<int32_t> ijk;       // P x 3 lattice integers
     std::vector<Row> rows;          // ny * nz
     DevBuf d_rows;
+    // tables made on first use, by any Hamiltonian on this mesh: made and
+    // looked up under the lock; an entry does not change or move once made
+    std::mutex mu;
     // tile lists keyed by (TX, TY, zseg): device tiles and their count
     std::map<std::tuple<int, int, int>, std::pair<DevBuf, int>> tiles;
     std::map<std::tuple<int, int, int>, std::vector<Tile>> tiles_host;   // the same lists on the host
@@ -303,7 +307,9 @@ void build_rows(rsg_mesh m, int64_t r2max) {
 
 // Tiles of TX x TY columns; each keeps only the planes where one of its rows
 // meets its x range, split into segments of zseg planes.
-rsg_status get_tiles(rsg_mesh m, int TX, int TY, int zseg, const Tile **out, int *count) {
+rsg_status get_tiles(rsg_mesh m, int TX, int TY, int zseg, const Tile **out, int *count,
+                     const std::vector<Tile> **host = nullptr) {
+    std::lock_guard<std::mutex> lock(m->mu);
     auto key = std::make_tuple(TX, TY, zseg);
     auto it = m->tiles.find(key);
     if (it == m->tiles.end()) {
@@ -372,6 +378,7 @@ rsg_status get_tiles(rsg_mesh m, int TX, int TY, int zseg, const Tile **out, int
     }
     *out = it->second.first.as<Tile>();
     *count = it->second.second;
+    if (host) *host = &m->tiles_host[key];
     return RSG_OK;
 }
 
@@ -445,6 +452,7 @@ bool default_c64(const TileCfg &c) {
 // Planes of every TX x TY column of tiles that holds mesh points, longest
 // first.
 const std::vector<int> &column_lengths(rsg_mesh m, int TX, int TY) {
+    std::lock_guard<std::mutex> lock(m->mu);
     auto it = m->col_len.find({TX, TY});
     if (it != m->col_len.end()) return it->second;
     const int ntx = (m->nx + TX - 1) / TX, nty = (m->ny + TY - 1) / TY;
@@ -670,6 +678,7 @@ struct Epi {
 bool has_potential(rsg_ham H) { return H->has_V || H->has_scaling; }
 
 rsg_status ensure_rows(rsg_mesh m) {
+    std::lock_guard<std::mutex> lock(m->mu);
     if (m->d_rows.p) return RSG_OK;
     CK(m->d_rows.upload(m->rows));
     return RSG_OK;
@@ -2832,7 +2841,8 @@ rsg_status batch_build_stages(rsg_batch b) {
         CK(b->w1[(size_t)i].ensure(bytes));
         const Tile *tiles = nullptr;
         int ntiles = 0;
-        CKS(get_tiles(m, kBatchNXR, kBatchTY, kBatchZseg, &tiles, &ntiles));
+        const std::vector<Tile> *host = nullptr;
+        CKS(get_tiles(m, kBatchNXR, kBatchTY, kBatchZseg, &tiles, &ntiles, &host));
         SysArgs &A = b->args[(size_t)i];
         A.vec[0] = nullptr;
         A.vec[1] = b->w0[(size_t)i].p;
@@ -2848,7 +2858,7 @@ rsg_status batch_build_stages(rsg_batch b) {
         for (int k = 0; k < 5; k++) A.w[k] = (float)(-0.5 * kFD[k] / (m->h * m->h));
         A.h3 = m->h * m->h * m->h;
         const int nch = (SV + kBatchCV - 1) / kBatchCV;
-        const std::vector<Tile> &ht = m->tiles_host[std::make_tuple(kBatchNXR, kBatchTY, kBatchZseg)];
+        const std::vector<Tile> &ht = *host;
         for (int t = 0; t < ntiles; t++)
             for (int c = 0; c < nch; c++) {
                 work.push_back(BWork{i, t, c, 0});
@@ -2937,8 +2947,9 @@ rsg_status batch_build_step(rsg_batch b) {
         batch_step_tile((int)ld, var, &TX, &TY);
         const Tile *tiles = nullptr;
         int ntiles = 0;
-        CKS(get_tiles(m, TX, TY, b->zseg, &tiles, &ntiles));
-        const std::vector<Tile> &ht = m->tiles_host[std::make_tuple(TX, TY, b->zseg)];
+        const std::vector<Tile> *host = nullptr;
+        CKS(get_tiles(m, TX, TY, b->zseg, &tiles, &ntiles, &host));
+        const std::vector<Tile> &ht = *host;
         SysArgs &A = b->args[(size_t)i];
         A.vec[0] = nullptr;
         A.vec[1] = b->w0[(size_t)i].p;
