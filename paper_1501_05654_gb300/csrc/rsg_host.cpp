@@ -177,6 +177,11 @@ struct rsg_mesh_s {
     std::map<std::tuple<int, int, int>, std::pair<DevBuf, int>> tiles;
     std::map<std::tuple<int, int, int>, std::vector<Tile>> tiles_host;   // the same lists on the host
     std::map<std::pair<int, int>, std::vector<int>> col_len;   // planes of every TX x TY column of tiles
+    // complex64: stencil kernel and segment length by (vectors per point,
+    // complex scaling, projectors); complex128: planes per block of the integer
+    // sums by vectors per point
+    std::map<std::tuple<int, bool, bool>, std::pair<int, int>> choice32;
+    std::map<int, int> choice64;
 };
 
 struct rsg_ham_s {
@@ -189,10 +194,6 @@ struct rsg_ham_s {
     double proj_norm = 0.0;            // bound on the non-local operator: sum over atoms of sum |h_ij|
     TileCfg cfg;
     bool force_kernel = false;   // set when the caller chose the kernel explicitly
-    // complex64: the kernel and segment length chosen per (vectors per point,
-    // complex scaling, projectors) in the default configuration; complex128:
-    // the sums and planes per block of kernel 1, per vectors per point
-    std::map<std::tuple<int, bool, bool>, TileCfg> auto_cfg;
     int last_kernel = -1;        // stencil kernel of the last application
     int last_zseg = 0;           // its planes per z segment (tiled kernels)
     int last_sum = 0;            // its planes per block with integer neighbour sums (complex128), 0: FP64 sums
@@ -539,27 +540,38 @@ double makespan(const std::vector<int> &col, int zs, int nch, int slots, int64_t
 // kernel, which all of these ran before: R = 10 sphere, 14 values a point:
 // 64 us (115); 96^3 x 16: 78 (168); 48^3 x 16: 19 (27); R = 14 sphere x 8:
 // 107 (173); 64^3 x 2: the plain kernel, 12.5 (21).
-TileCfg choose_c64(rsg_ham H, int SV) {
+// The choice is kept with the mesh.
+rsg_status choose_c64(rsg_ham H, int SV, std::pair<int, int> *choice) {
     const std::tuple<int, bool, bool> key(SV, H->has_scaling, H->pj.natoms > 0);
-    auto it = H->auto_cfg.find(key);
-    if (it != H->auto_cfg.end()) return it->second;
     rsg_mesh m = H->m;
-    TileCfg best = H->cfg, c5 = H->cfg;
+    {
+        std::lock_guard<std::mutex> lock(m->mu);
+        auto it = m->choice32.find(key);
+        if (it != m->choice32.end()) {
+            *choice = it->second;
+            return RSG_OK;
+        }
+    }
+    const TileCfg c7 = c64_config();
+    TileCfg c5 = c7;
     c5.kernel = 5;
-    c5.threads = 192;
-    c5.stages = 3;
-    c5.sync = 0;
+    std::pair<int, int> best(7, c7.zseg);
+    auto keep = [&]() {
+        std::lock_guard<std::mutex> lock(m->mu);
+        *choice = m->choice32[key] = best;
+        return RSG_OK;
+    };
     const int nch7 = (SV + 7) / 8, nch5 = (SV + 1) / 2;
     const bool narrow = SV % 8 != 0 && SV < 20, nl = H->pj.natoms > 0;
     int tx7, ty7, tx5, ty5;
-    block_shape(H->cfg, SV, &tx7, &ty7);
+    block_shape(c7, SV, &tx7, &ty7);
     block_shape(c5, SV, &tx5, &ty5);
     if (!narrow) {
         // enough blocks without a cut: nothing to choose
         const Tile *tiles = nullptr;
         int nt = 0;
-        if (get_tiles(m, tx7, ty7, best.zseg, &tiles, &nt) != RSG_OK || (int64_t)nt * nch7 >= 4 * 152)
-            return H->auto_cfg[key] = best;
+        CKS(get_tiles(m, tx7, ty7, c7.zseg, &tiles, &nt));
+        if ((int64_t)nt * nch7 >= 4 * 152) return keep();
     }
     const std::vector<int> &col7 = column_lengths(m, tx7, ty7), none;
     const std::vector<int> &col5 = SV % 8 != 0 ? column_lengths(m, tx5, ty5) : none;
@@ -575,19 +587,16 @@ TileCfg choose_c64(rsg_ham H, int SV) {
     };
     // without a cut: kernel 7, kernel 5 for narrow rows with a partly empty
     // chunk, the plain kernel where that leaves SMs without a block
-    double cost = narrow ? time5(150) : time7(best.zseg);
-    if (narrow) {
-        best = c5;
-        best.zseg = 150;
-    }
+    double cost = narrow ? time5(150) : time7(c7.zseg);
+    if (narrow) best = {5, 150};
     if (n < (narrow ? 304 : 152)) {
-        best.kernel = 1;
+        best.first = 1;
         cost = plain;
     }
     cost *= 0.92;   // the fit is good to a few percent: change for a clear gain only
     if (plain < cost) {
         cost = plain;
-        best.kernel = 1;
+        best.first = 1;
     }
     int last = 0;
     for (int zs : {190, 150, 96, 64, 48, 32, 24, 16, 12, 8}) {
@@ -596,17 +605,15 @@ TileCfg choose_c64(rsg_ham H, int SV) {
         const double t7 = time7(zs, cost);
         if (t7 < cost) {
             cost = t7;
-            best = H->cfg;
-            best.zseg = zs;
+            best = {7, zs};
         }
         const double t5 = SV % 8 != 0 && zs <= 150 ? time5(zs, cost) : cost;
         if (t5 < cost) {
             cost = t5;
-            best = c5;
-            best.zseg = zs;
+            best = {5, zs};
         }
     }
-    return H->auto_cfg[key] = best;
+    return keep();
 }
 
 // complex128: planes per block of the integer-sum kernel, or 0 for FP64 sums,
@@ -617,27 +624,29 @@ TileCfg choose_c64(rsg_ham H, int SV) {
 // R = 5 sphere x 5: 51 and 49; 32^3 x 4: 21 and 17; 61^3 x 8: 234 and 131 (8
 // planes a block; 148 with 32); 96^3 x 3: 325 and 179.
 int choose_c128(rsg_ham H, int SV) {
-    const std::tuple<int, bool, bool> key(SV, false, false);
-    auto it = H->auto_cfg.find(key);
-    if (it != H->auto_cfg.end()) return it->second.sum_zs;
+    rsg_mesh m = H->m;
+    {
+        std::lock_guard<std::mutex> lock(m->mu);
+        auto it = m->choice64.find(SV);
+        if (it != m->choice64.end()) return it->second;
+    }
     int tx, ty;
     sum64_shape(SV, &tx, &ty);
-    const std::vector<int> &col = column_lengths(H->m, tx, ty);
+    const std::vector<int> &col = column_lengths(m, tx, ty);
     const int ns = sum64_states(SV), nch = (SV + ns - 1) / ns;
-    TileCfg best = H->cfg;
-    best.sum_zs = 0;
-    double cost = 0.95 * (6.0 + 125e-6 * (double)H->m->P * SV);
+    int best = 0;
+    double cost = 0.95 * (6.0 + 125e-6 * (double)m->P * SV);
     for (int zs : {32, 24, 16, 12, 8, 6, 4, 3, 2, 1}) {
         int64_t n = 0;
         const double mk = makespan(col, zs, nch, 152, &n, 5, 1, (cost - 3.0) / (2.55 / 5));
         const double t = 3.0 + std::max(2.55 / 5 * mk, 3.2 * (col.empty() ? 0 : std::min(zs, col[0])));
         if (t < cost) {
             cost = t;
-            best.sum_zs = zs;
+            best = zs;
         }
     }
-    H->auto_cfg[key] = best;
-    return best.sum_zs;
+    std::lock_guard<std::mutex> lock(m->mu);
+    return m->choice64[SV] = best;
 }
 
 // ------------------------------------------------------------ checks ----
@@ -771,7 +780,17 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
     const int ldc_v = SV * (int)(16 / cbytes(H->dtype));
     const bool chosen = H->dtype == RSG_C64 && !H->force_kernel && !ep.fixed_kernel && !ep.twocol &&
                         m->bc == RSG_BC_ZERO && default_c64(H->cfg);
-    if (chosen) cfg = choose_c64(H, SV);
+    if (chosen) {
+        std::pair<int, int> choice;
+        CKS(choose_c64(H, SV, &choice));
+        cfg.kernel = choice.first;
+        cfg.zseg = choice.second;
+        if (cfg.kernel == 5) {
+            cfg.threads = 192;
+            cfg.stages = 3;
+            cfg.sync = 0;
+        }
+    }
     // kernel 7 moves 16-value chunks of each point row: blocks whose rows are
     // narrow or end in a mostly empty chunk take the register-blocked kernel
     // in its default shape unless kernel 7 was chosen explicitly; complex
