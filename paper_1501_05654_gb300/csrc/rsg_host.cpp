@@ -194,6 +194,7 @@ struct rsg_ham_s {
     double proj_norm = 0.0;            // bound on the non-local operator: sum over atoms of sum |h_ij|
     TileCfg cfg;
     bool force_kernel = false;   // set when the caller chose the kernel explicitly
+    bool shape_set = false;      // set when the caller chose a tile shape, even the default one
     int last_kernel = -1;        // stencil kernel of the last application
     int last_zseg = 0;           // its planes per z segment (tiled kernels)
     int last_sum = 0;            // its planes per block with integer neighbour sums (complex128), 0: FP64 sums
@@ -443,11 +444,6 @@ TileCfg c64_config() {
     c.zseg = 190;
     c.stages = 3;
     return c;
-}
-bool default_c64(const TileCfg &c) {
-    const TileCfg d = c64_config();
-    return c.kernel == d.kernel && c.wty == d.wty && c.npw == d.npw && c.threads == d.threads && c.zseg == d.zseg &&
-           c.stages == d.stages && c.sync == d.sync;
 }
 
 // Planes of every TX x TY column of tiles that holds mesh points, longest
@@ -779,7 +775,7 @@ rsg_status apply_t(rsg_ham H, const void *in, void *out, int SV, double eps, con
     TileCfg cfg = H->cfg;
     const int ldc_v = SV * (int)(16 / cbytes(H->dtype));
     const bool chosen = H->dtype == RSG_C64 && !H->force_kernel && !ep.fixed_kernel && !ep.twocol &&
-                        m->bc == RSG_BC_ZERO && default_c64(H->cfg);
+                        m->bc == RSG_BC_ZERO && !H->shape_set;
     if (chosen) {
         std::pair<int, int> choice;
         CKS(choose_c64(H, SV, &choice));
@@ -1359,6 +1355,8 @@ rsg_status rsg_ham_set_option(rsg_ham H, const char *key, int64_t value) {
     else if (k == "stages" && value >= 3 && value <= 5) H->cfg.stages = (int)value;
     else if (k == "blocks_per_sm" && (value == 2 || value == 3)) H->cfg.blocks_per_sm = (int)value;
     else return fail(RSG_ERR_ARG, "unknown option or value: %s=%lld", key, (long long)value);
+    if (k == "zseg" || k == "wide_ty" || k == "producers" || k == "threads" || k == "sync" || k == "stages")
+        H->shape_set = true;
     return RSG_OK;
 }
 
