@@ -1060,8 +1060,6 @@ std::vector<R> cast_vec(const std::vector<double> &v) {
     return std::vector<R>(v.begin(), v.end());
 }
 
-const int kChunk = 512;   // sphere entries per projector-dot block
-
 }  // namespace
 
 namespace rsg {
@@ -1451,7 +1449,7 @@ rsg_status rsg_field_set(rsg_ham H, double eps, const double dir[3]) {
 
 // Device tables of a projector set from its entry list: entry q is point
 // q_pt[q] of atom q_atom[q] with the npmax values q_p[q * npmax + i]; the
-// entries of each atom are contiguous and cut into chunks of at most kChunk
+// entries of each atom are contiguous and cut into chunks of at most kProjChunk
 // (ch_atom, ch_q0, ch_q1; atom_ch0 = per-atom prefix of chunks); hm holds the
 // zero-padded npmax x npmax coupling matrices.
 static rsg_status upload_projectors(rsg_ham H, int natoms, int npmax, const std::vector<int32_t> &q_pt,
@@ -1583,10 +1581,10 @@ rsg_status rsg_projectors_set(rsg_ham H, int natoms, const double *centres, cons
             if (nrm > 0)
                 for (size_t q = q_begin; q < q_end; q++) q_p[q * npmax + i] /= nrm;
         }
-        for (size_t q0 = q_begin; q0 < q_end; q0 += kChunk) {
+        for (size_t q0 = q_begin; q0 < q_end; q0 += kProjChunk) {
             ch_atom.push_back(a);
             ch_q0.push_back((int32_t)q0);
-            ch_q1.push_back((int32_t)std::min(q_end, q0 + kChunk));
+            ch_q1.push_back((int32_t)std::min(q_end, q0 + kProjChunk));
         }
         atom_ch0.push_back((int32_t)ch_q0.size());
         for (int i = 0; i < np; i++)
@@ -1659,10 +1657,10 @@ rsg_status rsg_projectors_set_raw(rsg_ham H, int natoms, const int64_t *npts, co
         }
         for (size_t q = q_begin; q < q_pt.size(); q++) seen[(size_t)q_pt[q]] = 0;
         const size_t q_end = q_pt.size();
-        for (size_t q0 = q_begin; q0 < q_end; q0 += kChunk) {
+        for (size_t q0 = q_begin; q0 < q_end; q0 += kProjChunk) {
             ch_atom.push_back(a);
             ch_q0.push_back((int32_t)q0);
-            ch_q1.push_back((int32_t)std::min(q_end, q0 + kChunk));
+            ch_q1.push_back((int32_t)std::min(q_end, q0 + kProjChunk));
         }
         atom_ch0.push_back((int32_t)ch_q0.size());
         double hmax = 0.0;

@@ -156,6 +156,9 @@ inline int proj_slices(int SV) {
     const int bv = SV < 32 ? SV : 32;   // vector slices of the coefficient kernels: bv vectors each
     return (SV + bv - 1) / bv;
 }
+// sphere entries of a coefficient block at most: the host cuts the chunks, the
+// kernel's shared memory holds one
+constexpr int kProjChunk = 512;
 // chained: the launch may overlap the end of the kernel before it.
 template <typename R>
 cudaError_t launch_proj_coeffs(const void *u, int SV, const ProjDev &pj, double *partial, unsigned *counter,

@@ -889,7 +889,6 @@ cudaError_t launch_apply(const ApplyArgs<R> &a, const TileCfg &cfg, int ntiles, 
 // per vector used to add the lanes of one projector at a time: one atom, one
 // vector a point 48 to 18 us; R = 18 sphere, 32 atoms x 4
 // projectors, 64 states 51 to 44 us; 192^3, 64 x 9, 128 states 0.59 to 0.46 ms.
-constexpr int kDotChunk = 512;   // entries of a chunk (the host cuts them)
 template <typename R, int NP>
 __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__restrict__ u, int SV,
                                                   const int32_t *__restrict__ q_pt,
@@ -906,8 +905,8 @@ __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__res
     constexpr int NCOMP = 2 * V::NC;
     // projector values of the chunk, then the lane sums, then the atom's c
     __shared__ __align__(16) unsigned char sm[NP * NCOMP * 256 * sizeof(R)];
-    __shared__ int qs[kDotChunk];
-    static_assert(kDotChunk * NP * sizeof(R) <= sizeof(sm) && 2 * NP * 32 * V::NC * sizeof(double) <= sizeof(sm), "");
+    __shared__ int qs[kProjChunk];
+    static_assert(kProjChunk * NP * sizeof(R) <= sizeof(sm) && 2 * NP * 32 * V::NC * sizeof(double) <= sizeof(sm), "");
     R *qv = (R *)sm, *red = (R *)sm;
     double *cbuf = (double *)sm;   // c[i][s] of the slice (re, im)
     chain_begin();
