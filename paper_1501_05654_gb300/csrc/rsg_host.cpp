@@ -203,10 +203,10 @@ struct rsg_ham_s {
     int adj_merge = -1;          // adjoint: costate and recompute sweeps share launches (1), not (0), auto (-1)
     // projectors
     ProjDev pj;
-    DevBuf q_pt, q_atom, q_p, ch_atom, ch_q0, ch_q1, atom_ch0, hm, nl_ptr, nl_ent, u_pts, u_ptr, e_atom, e_p;
+    DevBuf q_pt, q_p, ch_atom, ch_q0, ch_q1, atom_ch0, hm, nl_ptr, u_pts, u_ptr, e_atom, e_p;
     DevBuf D, partial, pcnt;   // coefficients, their partial sums, per-atom completion counters
     // workspace
-    DevBuf w0, w1, red, G, W, Wc, drift, status, dots, M, ov, grad, Xd, Xdir;
+    DevBuf w0, w1, red, G, W, Wc, drift, status, dots, ov, grad, Xd, Xdir;
     DevBuf w2, cg;     // shifted solver: third work block, per-state scalars
     DevBuf mask;       // mask absorber M(r) (compute type), applied after each time step
     bool has_mask = false;
@@ -1468,7 +1468,6 @@ static rsg_status upload_projectors(rsg_ham H, int natoms, int npmax, const std:
         for (size_t q = 0; q < q_pt.size(); q++) nl_ent[(size_t)fill[(size_t)q_pt[q]]++] = (int32_t)q;
     }
     CK(H->q_pt.upload(q_pt));
-    CK(H->q_atom.upload(q_atom));
     if (H->dtype == RSG_C64)
         CK(H->q_p.upload(cast_vec<float>(q_p)));
     else
@@ -1479,7 +1478,6 @@ static rsg_status upload_projectors(rsg_ham H, int natoms, int npmax, const std:
     CK(H->atom_ch0.upload(atom_ch0));
     CK(H->hm.upload(hm));
     CK(H->nl_ptr.upload(nl_ptr));
-    CK(H->nl_ent.upload(nl_ent));
     std::vector<int32_t> u_pts, u_ptr(1, 0);
     for (int64_t p = 0; p < P; p++)
         if (nl_ptr[(size_t)p + 1] > nl_ptr[(size_t)p]) {
@@ -1508,7 +1506,6 @@ static rsg_status upload_projectors(rsg_ham H, int natoms, int npmax, const std:
     pj.nq = (int64_t)q_pt.size();
     pj.nchunks = (int)ch_q0.size();
     pj.q_pt = H->q_pt.as<int32_t>();
-    pj.q_atom = H->q_atom.as<int32_t>();
     pj.q_p = H->q_p.p;
     pj.chunk_atom = H->ch_atom.as<int32_t>();
     pj.chunk_q0 = H->ch_q0.as<int32_t>();
@@ -1516,7 +1513,6 @@ static rsg_status upload_projectors(rsg_ham H, int natoms, int npmax, const std:
     pj.atom_chunk0 = H->atom_ch0.as<int32_t>();
     pj.hm = H->hm.as<double>();
     pj.nl_ptr = H->nl_ptr.as<int32_t>();
-    pj.nl_ent = H->nl_ent.as<int32_t>();
     pj.nu = (int)u_pts.size();
     pj.u_pts = H->u_pts.as<int32_t>();
     pj.u_ptr = H->u_ptr.as<int32_t>();
@@ -2395,8 +2391,7 @@ rsg_status control_gradient_t(rsg_ham H, const void *psi0, const void *target, i
     }
     const int nb = norm_blocks(P);
     const int nba = adjoint_blocks(P);
-    CK(H->dots.ensure((size_t)std::max(20 * nb, nba) * sizeof(double) + 64 * sizeof(double)));
-    CK(H->M.ensure(32 * sizeof(double)));
+    CK(H->dots.ensure((size_t)std::max(2 * nb, nba) * sizeof(double)));
     CK(H->ov.ensure(2 * sizeof(double)));
     CK(H->grad.ensure((size_t)nsteps * sizeof(double) + 64));
     CK(cudaMemsetAsync(H->grad.p, 0, (size_t)nsteps * sizeof(double) + 64, st));
@@ -2885,8 +2880,6 @@ rsg_status batch_build_stages(rsg_batch b) {
         A.nu = pj.nu;
         if (pj.natoms > 0) {
             A.q_pt = pj.q_pt;
-            A.q_atom = pj.q_atom;
-            A.nl_ent = pj.nl_ent;
             A.chunk_q0 = pj.chunk_q0;
             A.chunk_q1 = pj.chunk_q1;
             A.atom_chunk0 = pj.atom_chunk0;
@@ -3002,8 +2995,6 @@ rsg_status batch_build_step(rsg_batch b) {
             if (pj.npmax != 1 && pj.npmax != 4 && pj.npmax != 9)
                 return fail(RSG_ERR_UNSUPPORTED, "system %d: %d projectors per atom", i, pj.npmax);
             A.q_pt = pj.q_pt;
-            A.q_atom = pj.q_atom;
-            A.nl_ent = pj.nl_ent;
             A.chunk_q0 = pj.chunk_q0;
             A.chunk_q1 = pj.chunk_q1;
             A.atom_chunk0 = pj.atom_chunk0;

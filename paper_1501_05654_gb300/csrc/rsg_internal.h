@@ -99,15 +99,14 @@ struct ProjDev {
     int64_t nq = 0;
     int nchunks = 0;
     int32_t *q_pt = nullptr;      // point of each entry
-    int32_t *q_atom = nullptr;
     void *q_p = nullptr;          // R values, nq * npmax
     int32_t *chunk_atom = nullptr, *chunk_q0 = nullptr, *chunk_q1 = nullptr;
     int32_t *atom_chunk0 = nullptr; // natoms+1 prefix of chunks per atom
     double *hm = nullptr;         // natoms * npmax * npmax (zero padded)
-    int32_t *nl_ptr = nullptr, *nl_ent = nullptr;
+    int32_t *nl_ptr = nullptr;
     int nu = 0;                    // points inside at least one sphere
     int32_t *u_pts = nullptr, *u_ptr = nullptr;   // those points and their CSR rows
-    int32_t *e_atom = nullptr;     // per point-CSR entry: its atom (= q_atom[nl_ent[e]])
+    int32_t *e_atom = nullptr;     // per point-CSR entry: its atom
     void *e_p = nullptr;           // per point-CSR entry: its npmax projector values
 };
 
@@ -163,12 +162,6 @@ constexpr int kProjChunk = 512;
 template <typename R>
 cudaError_t launch_proj_coeffs(const void *u, int SV, const ProjDev &pj, double *partial, unsigned *counter,
                                double h3, void *D, bool chained, cudaStream_t st);
-template <typename R>
-cudaError_t launch_proj_dot(const void *u, int SV, const ProjDev &pj, double *partial,
-                            cudaStream_t st);
-template <typename R>
-cudaError_t launch_proj_reduce(const double *partial, int SV, const ProjDev &pj,
-                               double h3, void *D, cudaStream_t st);
 // out += alpha * (projector terms), acc += gamma * alpha * (same), over the
 // union points, reading the point-major entry copies (pj.e_atom, pj.e_p)
 template <typename R>
@@ -231,12 +224,6 @@ template <typename R>
 cudaError_t launch_norms(const void *psi, int64_t P, int ld, int S, double h3,
                          double *partial, int nblk, double *out, cudaStream_t st);
 int norm_blocks(int64_t P);
-// Inner products for the adjoint: out[j*4+i] = h3 sum_p conj(b_j) x_p a_i for
-// j + i <= 3 (complex double); b_j, a_i are P-vectors (S = 1, ld = 1 or 2).
-template <typename R>
-cudaError_t launch_adjoint_dots(const void *const *b, const void *const *a, int64_t P, int ld,
-                                const R *X, double h3, double *partial, int nblk,
-                                double *out, cudaStream_t st);
 // Fused adjoint inner products + reduction + grad_k update (one launch);
 // counter (device, zero on entry) is reset by the kernel.  ldb, lda: row
 // lengths of the b and the a blocks.
@@ -249,18 +236,10 @@ int adjoint_blocks(int64_t P);   // nblk of launch_adjoint_grad
 template <typename R>
 cudaError_t launch_overlap(const void *f, const void *g, int64_t P, int ld, double h3,
                            double *partial, int nblk, double *out, cudaStream_t st);
-// y = a * x (+ y if accumulate), complex scalar a given as device double[2]
-// or host values; one state vector or a whole block (n complex values).
-template <typename R>
-cudaError_t launch_axpby(const void *x, void *y, int64_t n, double ar, double ai,
-                         double br, double bi, cudaStream_t st);
 // y = x * (a[0] + i a[1]) where a is a DEVICE complex double (graph friendly)
 template <typename R>
 cudaError_t launch_scale_dev(const void *x, void *y, int64_t n, const double *a,
                              cudaStream_t st);
-// grad[k] += 2 Re( -i tau * sum_n 1/n! sum_j M[j][n-1-j] )  (device)
-cudaError_t launch_grad_accum(const double *M, double tau, double *grad_k,
-                              cudaStream_t st);
 
 // ---- batches of independent complex64 systems (rsg_kernels.cu) ----
 // Per-system arguments, resident on the device.  vec[] = {psi, w0, w1}: the
@@ -274,7 +253,7 @@ struct SysArgs {
     const float *V;
     float w[5];
     int natoms, npmax, nu;
-    const int32_t *q_pt, *q_atom, *nl_ent, *chunk_q0, *chunk_q1, *atom_chunk0, *u_pts, *u_ptr, *e_atom;
+    const int32_t *q_pt, *chunk_q0, *chunk_q1, *atom_chunk0, *u_pts, *u_ptr, *e_atom;
     const float *q_p, *e_p;
     const double *hm;
     float *D;

@@ -26,7 +26,7 @@
 //                   run k_apply_sum64, rsg_sum64.cu).
 //   k_proj_dot      partial sums of <p_ai|u_s> over sphere chunks (FP32
 //                   products and partial sums for complex64, FP64 across
-//                   chunks), k_proj_reduce: h^3 sum over chunks, times h_a.
+//                   chunks); an atom's last block: h^3 sum, times h_a.
 #include <cuda.h>
 
 #include "rsg_async.cuh"
@@ -98,15 +98,6 @@ __device__ __forceinline__ void finish_point(const ApplyArgs<R> &a, int64_t idx,
     using T = typename VT<R>::T;
     const T b = a.base != nullptr ? ((const T *)a.base)[idx * a.SV + v] : VT<R>::zero();
     finish_point<R>(a, idx, x, y, z, v, center, acc, a.V[idx], b, load_projectors<R>(a, idx));
-}
-
-// Value of vector v at bbox (x, row) or zero outside the mesh.
-template <typename R>
-__device__ __forceinline__ typename VT<R>::T row_value(const typename VT<R>::T *in,
-                                                       const Row &rw, int x, int SV, int v) {
-    if (x >= rw.xmin && x <= rw.xmax)
-        return VT<R>::ldg(in + ((int64_t)rw.start + (x - rw.xmin)) * SV + v);
-    return VT<R>::zero();
 }
 
 // --------------------------------------------------------- z-marching ---
@@ -875,11 +866,10 @@ cudaError_t launch_apply(const ApplyArgs<R> &a, const TileCfg &cfg, int ntiles, 
 // Block: (BV vectors) x (PL point lanes).  Chunk c covers entries [q0, q1)
 // of one atom.  partial[((c * npmax + i) * SV + v) * 2 * NC + comp] (FP64).
 //
-// With counter != nullptr the coefficients are finished in the same launch:
-// after writing its partial sums a block counts itself done for its atom
-// (per vector slice blockIdx.y), and the last block of an atom sums the
-// atom's chunks in chunk order, scales by h^3 and applies h_a, exactly as
-// k_proj_reduce does, then resets the counter for the next launch.
+// The coefficients are finished in the same launch: after writing its partial
+// sums a block counts itself done for its atom (per vector slice blockIdx.y),
+// and the last block of an atom sums the atom's chunks in chunk order, scales
+// by h^3 and applies h_a, then resets the counter for the next launch.
 //
 // The chunk's point indices and projector values are staged first, so that a
 // lane's state loads (UNR in flight) depend on nothing but shared memory; the
@@ -958,7 +948,6 @@ __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__res
         for (int l = 0; l < by; l++) s += (double)red[ij * 256 + l * bx + x];
         partial[(((int64_t)c * NP + ij / NCOMP) * SV + vv) * NCOMP + ij % NCOMP] = s;
     }
-    if (counter == nullptr) return;
     // the last block of this atom and vector slice finishes its coefficients
     __shared__ int last;
     __threadfence();
@@ -1007,12 +996,6 @@ __global__ void __launch_bounds__(256) k_proj_dot(const typename VT<R>::T *__res
 }
 
 template <typename R>
-cudaError_t launch_proj_dot(const void *u, int SV, const ProjDev &pj, double *partial,
-                            cudaStream_t st) {
-    return launch_proj_coeffs<R>(u, SV, pj, partial, nullptr, 0.0, nullptr, false, st);
-}
-
-template <typename R>
 cudaError_t launch_proj_coeffs(const void *u, int SV, const ProjDev &pj, double *partial, unsigned *counter,
                                double h3, void *D, bool chained, cudaStream_t st) {
     if (pj.natoms == 0 || pj.nchunks == 0) return cudaSuccess;
@@ -1034,42 +1017,6 @@ cudaError_t launch_proj_coeffs(const void *u, int SV, const ProjDev &pj, double 
     default: return cudaErrorInvalidValue;
     }
 #undef RSG_PROJ_DOT
-}
-
-// One thread per (atom, complex column s).  c_i = h3 * sum over the atom's
-// chunks; D[a, i, s] = sum_j h_a[i][j] c_j, stored in the compute type.
-template <typename R>
-__global__ void k_proj_reduce(const double *__restrict__ partial, int SV, int natoms, int npmax,
-                              const int32_t *__restrict__ atom_chunk0,
-                              const double *__restrict__ hm, double h3, R *__restrict__ D) {
-    constexpr int NC = VT<R>::NC;
-    const int ldc = SV * NC;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= natoms * ldc) return;
-    const int a = t / ldc, s = t % ldc;
-    double cr[9], ci[9];
-    for (int i = 0; i < npmax; i++) {
-        double sr = 0.0, si = 0.0;
-#pragma unroll 4
-        for (int c = atom_chunk0[a]; c < atom_chunk0[a + 1]; c++) {
-            const double *p = partial + (((int64_t)c * npmax + i) * ldc + s) * 2;
-            sr += p[0];
-            si += p[1];
-        }
-        cr[i] = h3 * sr;
-        ci[i] = h3 * si;
-    }
-    for (int i = 0; i < npmax; i++) {
-        double dr = 0.0, di = 0.0;
-        for (int j = 0; j < npmax; j++) {
-            const double hij = hm[((int64_t)a * npmax + i) * npmax + j];
-            dr += hij * cr[j];
-            di += hij * ci[j];
-        }
-        R *dst = D + (((int64_t)a * npmax + i) * ldc + s) * 2;
-        dst[0] = (R)dr;
-        dst[1] = (R)di;
-    }
 }
 
 // Projector terms of H u added to an already written result:
@@ -1168,16 +1115,6 @@ cudaError_t launch_proj_scatter(const ApplyArgs<R> &a, const ProjDev &pj, cudaSt
     default: return cudaErrorInvalidValue;
     }
 #undef RSG_PROJ_SCATTER
-    return cudaGetLastError();
-}
-
-template <typename R>
-cudaError_t launch_proj_reduce(const double *partial, int SV, const ProjDev &pj, double h3,
-                               void *D, cudaStream_t st) {
-    if (pj.natoms == 0) return cudaSuccess;
-    const int n = pj.natoms * SV * VT<R>::NC;
-    k_proj_reduce<R><<<(n + 127) / 128, 128, 0, st>>>(partial, SV, pj.natoms, pj.npmax,
-                                                       pj.atom_chunk0, pj.hm, h3, (R *)D);
     return cudaGetLastError();
 }
 
@@ -2049,10 +1986,8 @@ template cudaError_t launch_apply_rowtma<float>(const ApplyArgs<float> &, const 
 template cudaError_t launch_apply_tma<float>(const ApplyArgs<float> &, const TileCfg &, int, cudaStream_t, bool *);
 template cudaError_t launch_apply<float>(const ApplyArgs<float> &, const TileCfg &, int, cudaStream_t);
 template cudaError_t launch_apply_naive_odd<float>(const ApplyArgs<float> &, cudaStream_t);
-template cudaError_t launch_proj_dot<float>(const void *, int, const ProjDev &, double *, cudaStream_t);
 template cudaError_t launch_proj_coeffs<float>(const void *, int, const ProjDev &, double *, unsigned *, double,
                                                void *, bool, cudaStream_t);
-template cudaError_t launch_proj_reduce<float>(const double *, int, const ProjDev &, double, void *, cudaStream_t);
 template cudaError_t launch_proj_scatter<float>(const ApplyArgs<float> &, const ProjDev &, cudaStream_t);
 #endif
 #ifndef RSG_ONLY_FLOAT
@@ -2060,10 +1995,8 @@ template cudaError_t launch_apply_tma<double>(const ApplyArgs<double> &, const T
 template cudaError_t launch_apply_rowtma<double>(const ApplyArgs<double> &, const TileCfg &, int, cudaStream_t, bool *);
 template cudaError_t launch_apply<double>(const ApplyArgs<double> &, const TileCfg &, int, cudaStream_t);
 template cudaError_t launch_apply_naive_odd<double>(const ApplyArgs<double> &, cudaStream_t);
-template cudaError_t launch_proj_dot<double>(const void *, int, const ProjDev &, double *, cudaStream_t);
 template cudaError_t launch_proj_coeffs<double>(const void *, int, const ProjDev &, double *, unsigned *, double,
                                                 void *, bool, cudaStream_t);
-template cudaError_t launch_proj_reduce<double>(const double *, int, const ProjDev &, double, void *, cudaStream_t);
 template cudaError_t launch_proj_scatter<double>(const ApplyArgs<double> &, const ProjDev &, cudaStream_t);
 #endif
 

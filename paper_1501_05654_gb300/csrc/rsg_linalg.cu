@@ -370,63 +370,20 @@ __global__ void __launch_bounds__(256) k_norms(const R *__restrict__ psi, int64_
 template <typename R>
 cudaError_t launch_norms(const void *psi, int64_t P, int ld, int S, double h3, double *partial,
                          int nblk, double *out, cudaStream_t st) {
-    if constexpr (sizeof(R) == 4) return launch_norms_c64(psi, P, ld, S, h3, partial, nblk, out, st);
-    const int bx = S < 32 ? S : 32;
-    k_norms<R><<<nblk, dim3(bx, 256 / bx), 0, st>>>((const R *)psi, P, ld, S, partial, nblk);
-    return launch_sum_blocks(partial, nblk, S, h3, out, st);
-}
-
-// Ten inner products <b_j| X |a_i>, j + i <= 3, for the adjoint gradient.
-template <typename R>
-__global__ void __launch_bounds__(256) k_adjoint_dots(const R *b0, const R *b1, const R *b2,
-                                                      const R *b3, const R *a0, const R *a1,
-                                                      const R *a2, const R *a3, int64_t P, int ld,
-                                                      const R *__restrict__ X,
-                                                      double *__restrict__ partial, int nblk) {
-    __shared__ double red[256];
-    const R *bb[4] = {b0, b1, b2, b3};
-    const R *aa[4] = {a0, a1, a2, a3};
-    double acc[20];
-#pragma unroll
-    for (int i = 0; i < 20; i++) acc[i] = 0.0;
-    const int64_t per = (P + nblk - 1) / nblk;
-    const int64_t p0 = blockIdx.x * per;
-    const int64_t p1 = p0 + per < P ? p0 + per : P;
-    for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        double br[4], bi[4], ar[4], ai[4];
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            ld_c(bb[j] + p * ld * 2, br[j], bi[j]);
-            ld_c(aa[j] + p * ld * 2, ar[j], ai[j]);
-        }
-        const double x = (double)X[p];
-        int k = 0;
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-#pragma unroll
-            for (int i = 0; i + j <= 3; i++) {
-                // conj(b) * x * a
-                acc[2 * k] += x * (br[j] * ar[i] + bi[j] * ai[i]);
-                acc[2 * k + 1] += x * (br[j] * ai[i] - bi[j] * ar[i]);
-                k++;
-            }
-    }
-    for (int k = 0; k < 20; k++) {
-        red[threadIdx.x] = acc[k];
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) partial[(int64_t)blockIdx.x * 20 + k] = red[0];
-        __syncthreads();
+    if constexpr (sizeof(R) == 4) {
+        return launch_norms_c64(psi, P, ld, S, h3, partial, nblk, out, st);
+    } else {
+        const int bx = S < 32 ? S : 32;
+        k_norms<R><<<nblk, dim3(bx, 256 / bx), 0, st>>>((const R *)psi, P, ld, S, partial, nblk);
+        return launch_sum_blocks(partial, nblk, S, h3, out, st);
     }
 }
 
-// Fused form for the control gradient: the same per-block partial sums, then
-// the last block to finish (ticket counter) sums the partials in block order
-// and adds 2 Re(-i tau sum_n 1/n! sum_j M[j][n-1-j]) = 2 tau Im(...) to grad_k.
-// The counter is left at zero for the next call.
+// Adjoint gradient of one exponential: per-block partial sums of the inner
+// products M[j][i] = h^3 <b_j| X |a_i> that enter it, then the last block to
+// finish (ticket counter) sums the partials in block order and adds
+// 2 Re(-i tau sum_n 1/n! sum_j M[j][n-1-j]) = 2 tau Im(...) to grad_k.  The
+// counter is left at zero for the next call.
 template <typename R>
 __global__ void __launch_bounds__(256) k_adjoint_grad(const R *b0, const R *b1, const R *b2, const R *b3,
                                                       const R *a0, const R *a1, const R *a2, const R *a3,
@@ -515,37 +472,6 @@ cudaError_t launch_adjoint_grad(const void *const *b, const void *const *a, int6
                           (const R *)a[3], P, ldb, lda, X, h3, tau, partial, nblk, counter, grad_k);
 }
 
-// Expand the 10 packed values into out[j*4+i] (complex double), zero elsewhere.
-__global__ void k_adjoint_finish(const double *packed, double *out) {
-    if (threadIdx.x != 0) return;
-    int k = 0;
-    for (int j = 0; j < 4; j++)
-        for (int i = 0; i < 4; i++) {
-            if (i + j <= 3) {
-                out[(j * 4 + i) * 2] = packed[2 * k];
-                out[(j * 4 + i) * 2 + 1] = packed[2 * k + 1];
-                k++;
-            } else {
-                out[(j * 4 + i) * 2] = 0.0;
-                out[(j * 4 + i) * 2 + 1] = 0.0;
-            }
-        }
-}
-
-template <typename R>
-cudaError_t launch_adjoint_dots(const void *const *b, const void *const *a, int64_t P, int ld,
-                                const R *X, double h3, double *partial, int nblk, double *out,
-                                cudaStream_t st) {
-    k_adjoint_dots<R><<<nblk, 256, 0, st>>>((const R *)b[0], (const R *)b[1], (const R *)b[2],
-                                             (const R *)b[3], (const R *)a[0], (const R *)a[1],
-                                             (const R *)a[2], (const R *)a[3], P, ld, X, partial,
-                                             nblk);
-    double *packed = partial + (int64_t)nblk * 20;
-    if (cudaError_t e = launch_sum_blocks(partial, nblk, 20, h3, packed, st)) return e;
-    k_adjoint_finish<<<1, 32, 0, st>>>(packed, out);
-    return cudaGetLastError();
-}
-
 // h3 * sum_p conj(f_p) g_p for column 0 of two (P, ld) blocks.
 template <typename R>
 __global__ void __launch_bounds__(256) k_overlap(const R *__restrict__ f, const R *__restrict__ g,
@@ -586,29 +512,6 @@ cudaError_t launch_overlap(const void *f, const void *g, int64_t P, int ld, doub
     return launch_sum_blocks(partial, nblk, 2, h3, out, st);
 }
 
-// y = a x + b y over n complex values
-template <typename R>
-__global__ void k_axpby(const R *__restrict__ x, R *__restrict__ y, int64_t n, double ar, double ai,
-                        double br, double bi) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const double xr = x[2 * i], xi = x[2 * i + 1];
-        const double yr = y[2 * i], yi = y[2 * i + 1];
-        y[2 * i] = (R)(ar * xr - ai * xi + br * yr - bi * yi);
-        y[2 * i + 1] = (R)(ar * xi + ai * xr + br * yi + bi * yr);
-    }
-}
-
-template <typename R>
-cudaError_t launch_axpby(const void *x, void *y, int64_t n, double ar, double ai, double br,
-                         double bi, cudaStream_t st) {
-    int64_t nb = (n + 255) / 256;
-    if (nb > 152 * 16) nb = 152 * 16;
-    if (nb < 1) nb = 1;
-    k_axpby<R><<<(unsigned)nb, 256, 0, st>>>((const R *)x, (R *)y, n, ar, ai, br, bi);
-    return cudaGetLastError();
-}
-
 template <typename R>
 __global__ void k_scale_dev(const R *__restrict__ x, R *__restrict__ y, int64_t n,
                             const double *__restrict__ a) {
@@ -630,26 +533,6 @@ cudaError_t launch_scale_dev(const void *x, void *y, int64_t n, const double *a,
     return cudaGetLastError();
 }
 
-// grad_k += 2 Re( -i tau * sum_{n=1..4} 1/n! sum_{j<n} M[j][n-1-j] )
-__global__ void k_grad_accum(const double *M, double tau, double *g) {
-    if (threadIdx.x != 0) return;
-    const double invf[5] = {1.0, 1.0, 0.5, 1.0 / 6.0, 1.0 / 24.0};
-    double sr = 0.0, si = 0.0;
-    for (int n = 1; n <= 4; n++)
-        for (int j = 0; j < n; j++) {
-            const int i = n - 1 - j;
-            sr += invf[n] * M[(j * 4 + i) * 2];
-            si += invf[n] * M[(j * 4 + i) * 2 + 1];
-        }
-    // Re(-i tau (sr + i si)) = tau * si
-    *g += 2.0 * tau * si;
-}
-
-cudaError_t launch_grad_accum(const double *M, double tau, double *grad_k, cudaStream_t st) {
-    k_grad_accum<<<1, 32, 0, st>>>(M, tau, grad_k);
-    return cudaGetLastError();
-}
-
 #define RSG_INST(R)                                                                               \
     template cudaError_t launch_rotate<R>(void *, int64_t, int, int, const double *, cudaStream_t);  \
     template cudaError_t launch_resid<R>(const void *, const void *, int64_t, int, int, const double *, \
@@ -663,17 +546,12 @@ cudaError_t launch_grad_accum(const double *M, double tau, double *grad_k, cudaS
                                              cudaStream_t);                                          \
     template cudaError_t launch_norms<R>(const void *, int64_t, int, int, double, double *, int,     \
                                          double *, cudaStream_t);                                    \
-    template cudaError_t launch_adjoint_dots<R>(const void *const *, const void *const *, int64_t,   \
-                                                int, const R *, double, double *, int, double *,     \
-                                                cudaStream_t);                                       \
     template cudaError_t launch_adjoint_grad<R>(const void *const *, const void *const *, int64_t, int, \
                                                 int, const R *, double, double, double *, int,         \
                                                 unsigned *,                                            \
                                                 double *, cudaStream_t);                               \
     template cudaError_t launch_overlap<R>(const void *, const void *, int64_t, int, double,         \
                                            double *, int, double *, cudaStream_t);                   \
-    template cudaError_t launch_axpby<R>(const void *, void *, int64_t, double, double, double,      \
-                                         double, cudaStream_t);                                      \
     template cudaError_t launch_scale_dev<R>(const void *, void *, int64_t, const double *,         \
                                              cudaStream_t);
 RSG_INST(float)

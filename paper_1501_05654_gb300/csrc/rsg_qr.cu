@@ -952,12 +952,10 @@ cudaError_t launch_tri_apply_c64(void *psi, int64_t P, int ld, int S, const doub
     }
 }
 
-#define RSG_INST_QR(R)                                                                                        \
-    template cudaError_t launch_gram<R>(const void *, int64_t, int, int, double, double *, int, double *,     \
-                                        cudaStream_t);                                                        \
-    template cudaError_t launch_cross_gram<R>(const void *, const void *, int64_t, int, int, double, double *, \
-                                              int, double *, cudaStream_t);
-RSG_INST_QR(float)
-RSG_INST_QR(double)
+template cudaError_t launch_gram<double>(const void *, int64_t, int, int, double, double *, int, double *, cudaStream_t);
+template cudaError_t launch_cross_gram<float>(const void *, const void *, int64_t, int, int, double, double *, int,
+                                              double *, cudaStream_t);
+template cudaError_t launch_cross_gram<double>(const void *, const void *, int64_t, int, int, double, double *, int,
+                                               double *, cudaStream_t);
 
 }  // namespace rsg
