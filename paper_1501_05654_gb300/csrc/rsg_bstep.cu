@@ -256,11 +256,12 @@ __device__ int bs_stencil(const BStepArgs &A, int it, unsigned s_ring, unsigned 
         }
         int issued = 0;
         for (int j = j0; j <= j1; j++) {
-            if (*babort) break;
             const unsigned jg = J + (unsigned)(j - j0);
             const int s = (int)(jg % kBNS);
             const unsigned full = bar0 + 8 * s, empty = bar0 + 8 * (kBNS + s);
-            if (jg >= (unsigned)kBNS && !bs_wait(empty, (jg / kBNS - 1u) & 1u, babort)) break;
+            // a warp leaves as one: its other lanes would wait for the leavers below
+            const bool go = !*babort && (jg < (unsigned)kBNS || bs_wait(empty, (jg / kBNS - 1u) & 1u, babort));
+            if (!__all_sync(0xffffffffu, go)) break;
             const unsigned slot = s_ring + (unsigned)(s * kBSlot);
             unsigned vd = 0, zd = 0, zd2 = 0;
             int vp = 0, vn = 0, zn = 0, zn2 = 0;
@@ -393,7 +394,7 @@ __device__ int bs_stencil(const BStepArgs &A, int it, unsigned s_ring, unsigned 
         const unsigned jg = J + (unsigned)(j - j0);
         const int sl = (int)(jg % kBNS);
         const unsigned full = bar0 + 8 * sl, empty = bar0 + 8 * (kBNS + sl);
-        if (!bs_wait(full, (jg / kBNS) & 1u, babort)) break;
+        if (!__all_sync(0xffffffffu, bs_wait(full, (jg / kBNS) & 1u, babort))) break;
         if (j >= jc0 && j <= jc1 + 4) {
             const unsigned char *slotp = gring + (size_t)sl * kBSlot;
             float2 s[4], cen[4];
