@@ -541,8 +541,19 @@ class Batch:
             _lib.rsg_batch_destroy(self._h)
             self._h = None
 
+    def _check(self, psis):
+        """The library reads and writes P * padded_ld(S) values of every block."""
+        if len(psis) != len(self.hams):
+            raise ValueError(f"expected {len(self.hams)} state blocks, got {len(psis)}")
+        for i, (p, H, S) in enumerate(zip(psis, self.hams, self.S)):
+            ld = padded_ld(S, torch.complex64)
+            if not (isinstance(p, torch.Tensor) and p.is_cuda and p.dtype == torch.complex64 and p.is_contiguous()
+                    and p.numel() >= H.mesh.P * ld):
+                raise ValueError(f"block {i}: expected a contiguous cuda complex64 tensor of shape ({H.mesh.P}, {ld})")
+
     def propagate(self, psis, nsteps: int, dt: float, scheme: int = ETRS, gs_every: int = 0,
                   stream=None):
+        self._check(psis)
         ptrs = (C.c_void_p * len(psis))(*[p.data_ptr() for p in psis])
         _ck(load().rsg_batch_propagate(self._h, ptrs, int(nsteps), float(dt), int(scheme),
                                        int(gs_every), _stream(stream)))
@@ -558,6 +569,7 @@ class Batch:
     def autotune(self, psis, dt: float, scheme: int = ETRS, stream=None) -> float:
         """Choose launch mode, segment length and tile variants by timing
         steps on copies of psis; returns the best time per step in ms."""
+        self._check(psis)
         ptrs = (C.c_void_p * len(psis))(*[p.data_ptr() for p in psis])
         ms = C.c_double()
         _ck(load().rsg_batch_autotune(self._h, ptrs, float(dt), int(scheme), _stream(stream), C.byref(ms)))
