@@ -81,7 +81,17 @@ def peaks():
 
 # stencil kernel of each "kernel" option value (rsg_ham_get_option "last_kernel")
 KERNEL_NAMES = {0: "k_apply_staged", 1: "k_apply_naive", 2: "k_apply_zmarch", 3: "k_apply_tma",
-                4: "k_apply_rowtma", 5: "k_apply_quad", 7: "k_apply_wide"}   # 1 in complex128: k_apply_sum64 or k_apply_row64
+                4: "k_apply_rowtma", 5: "k_apply_quad", 7: "k_apply_wide"}
+
+
+def stencil_name(H):
+    """The stencil kernel of H's last application."""
+    k = H.get_option("last_kernel")
+    if k == 1 and str(H.dtype) == "torch.complex128":
+        return "k_apply_sum64" if H.get_option("last_sum_planes") > 0 else "k_apply_row64"
+    return KERNEL_NAMES.get(k, "unknown")
+
+
 # the files the dominant stencil kernel (k_apply_wide) is compiled from; the
 # public header it also includes holds only C declarations the kernel does
 # not use
@@ -400,7 +410,7 @@ def collect_headline_checks(H, mesh, psi_h, kname):
     torch.cuda.synchronize()
     chk["etrs_small"] = {"radius": 6.0, "wells": w6, "proj": p6, "lib_ijk": m6.ijk, "psi": x6.astype(np.complex128),
                          "out": t6.cpu().numpy().astype(np.complex128),
-                         "kernel": KERNEL_NAMES.get(H6.get_option("last_kernel"), "unknown")}
+                         "kernel": stencil_name(H6)}
     return chk
 
 
@@ -640,7 +650,7 @@ def extras(mesh, wells, proj, g, chk):
     ms5 = time_steps(None, x5, 3, lambda x: H5.propagate(x, 1, 0.01, scheme=rsg.ETRS, want_drift=False))
     k5_ms, _, k5_bytes, _ = H5.kernel_stats()
     H5.profile(False)
-    k5_name = KERNEL_NAMES.get(H5.get_option("last_kernel"), "unknown")
+    k5_name = stencil_name(H5)
     torch.cuda.synchronize()
     g0 = time.perf_counter()
     H5.orthonormalize(x5)
@@ -974,7 +984,7 @@ def main():
     peak, peak_kind = peaks()
     achieved = (k_bytes / k_n) / (k_ms / k_n * 1e-3) / 1e9 if k_n else None
     per_launch_bytes = k_bytes / k_n if k_n else None
-    kname = KERNEL_NAMES.get(H.get_option("last_kernel"), "unknown")
+    kname = stencil_name(H)
     traffic = traffic_record(kernel_hash(), kname)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
