@@ -616,9 +616,11 @@ rsg_status choose_c64(rsg_ham H, int SV, std::pair<int, int> *choice) {
 // by the smaller of two fitted times (us): FP64 sums 6 + 125e-6 per value; the
 // integer kernel 3 plus its schedule over the SMs at 2.55 a plane (two blocks
 // share an SM's issue slots; a block starts in a fifth of a plane), at least
-// 3.2 a plane for a block by itself.  24^3 x 1: 8.8 and 9.2 us (FP64 sums taken);
-// R = 5 sphere x 5: 51 and 49; 32^3 x 4: 21 and 17; 61^3 x 8: 234 and 131 (8
-// planes a block; 148 with 32); 96^3 x 3: 325 and 179.
+// 3.2 a plane for a block by itself.  The fit is to single applications.  In a
+// chain of steps (us an application, FP64 and integer sums): 16^3 x 1 3.9 and
+// 5.5 (FP64 taken); 24^3 x 1 4.2 and 6.9, 24^3 x 4 8.4 and 7.5, 32^3 x 4 16.9 and
+// 12.7, 61^3 x 8 209 and 121, 96^3 x 3 292 and 168 (integers taken in all five;
+// at 24^3 x 1 single applications take 8.8 and 9.2).
 int choose_c128(rsg_ham H, int SV) {
     rsg_mesh m = H->m;
     {

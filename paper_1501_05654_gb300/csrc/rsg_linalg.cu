@@ -1,7 +1,8 @@
 // FP64 reductions and small dense linear algebra on state blocks.
 //
-// Norms, Gram matrices, the Cholesky factor of the Gram matrix and its
-// inverse are kept in FP64 for both compute types (arXiv:1501.05654,
+// The Cholesky factor of the Gram matrix, its inverse and the sums over points
+// are FP64 for both compute types; complex64 norms and Gram matrices reach
+// them through short FP32 sums (rsg_qr.cu) (arXiv:1501.05654,
 // Sec. "Parallelization, optimizations and graphics processing units": real-time propagation preserves orthogonality, so the
 // states are re-orthonormalised only now and then; here Cholesky-QR, which
 // equals Gram-Schmidt in index order; the Gram matrices, the factor and the

@@ -1,5 +1,5 @@
-// Cholesky-QR of complex64 state blocks: FP64 norms, the Gram matrix, and the
-// triangular update (arXiv:1501.05654, Sec. "Parallelization, optimizations
+// Cholesky-QR of complex64 state blocks: norms to FP64 accuracy, the Gram
+// matrix, and the triangular update (arXiv:1501.05654, Sec. "Parallelization, optimizations
 // and graphics processing units": orthogonalisation of a group of states);
 // and the Gram matrices of FP64 accumulation shared with the eigensolver.
 //
