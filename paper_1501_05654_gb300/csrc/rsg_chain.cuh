@@ -8,8 +8,8 @@
 // before it touches a state, a coefficient or a counter.  Every thread of a
 // chained kernel calls chain_wait before it leaves, so it never completes
 // before its predecessor; a kernel launched without the attribute waits for
-// all of it.  32^3 x 4 complex128: 14.4 to 11.7 us per application; 48^3 x 16
-// with projectors 37 to 33 us.  Where it does not pay: the projector scatter
+// all of it.  32^3 x 4 complex128: 16.4 to 12.5 us per application; 48^3 x 16
+// with projectors 36.9 to 33.3 us.  Where it does not pay: the projector scatter
 // (its early blocks hold registers the stencil's last blocks need: 192^3 + 3%)
 // and the coefficients in front of the plain kernels (+15%) launch as usual.
 #pragma once
