@@ -10,7 +10,6 @@
 // off the inner loops: runs of FP32 sums are collected in short two-float sums
 // before they meet FP64.
 #include <algorithm>
-#include <type_traits>
 
 #include "rsg_async.cuh"
 #include "rsg_internal.h"
@@ -193,17 +192,36 @@ __global__ void __launch_bounds__(256) k_sum_herm(const double2 *__restrict__ pa
 // threads are several groups that share the staged points.  FP32 products
 // are summed in FP32 over runs of 8 points; kGHeld runs are collected in a
 // two-float sum (whose own rounding, below 2^-37 of its largest partial sum,
-// lies under the 2^-24 of the runs), which is added to an FP64 sum.  A block
-// in which such a sum leaves the FP32 range although its runs do not (squares
-// near 1e36) sums its points again, every run in FP64.  The points come as
+// lies under the 2^-24 of the runs), which is added to an FP64 sum.  An entry
+// whose two-float sums leave the FP32 range although its runs do not (squares
+// near 1e36) is summed again, every run in FP64.  The points come as
 // they lie (one 16-byte asynchronous copy per two states), double-buffered;
-// on the diagonal both operands are the same panel.  192^3 x 128 states: 19
+// on the diagonal both operands are the same panel.  192^3 x 128 states: 18
 // ms (108 ms when every run met two FP64 additions and conversions per value;
 // kGHeld = 64 adds 0.6 ms, one two-float sum for all of a block's points, of
-// less range and fewer bits, saves 2; FP64 sums in shared memory save nothing).
+// less range and fewer bits, saves 0.8; a second pass of the block instead of
+// the entry's own sums costs 0.6 by its code alone).
 // The point blocks are `nsub` pieces of the blocks of 4096 points or more
 // that gram_blocks names, cut at multiples of a run.
 constexpr int kGHeld = 128;   // runs in a two-float sum
+// One entry's sum again, every run added in FP64: `runs` runs of 8 points from
+// p on, then those `step` points further, up to p1.
+__device__ __noinline__ double2 gram_runs64(const float2 *x, const float2 *y, int64_t p, int64_t p1, int ld, int runs,
+                                            int step) {
+    double2 tot = make_double2(0.0, 0.0);
+    for (; p < p1; p += step)
+        for (int64_t r = p; r < p + 8 * runs && r < p1; r += 8) {
+            float2 f = make_float2(0.f, 0.f);
+            for (int64_t q = r; q < r + 8 && q < p1; q++) {
+                const float2 a = x[q * ld], b = y[q * ld];
+                f.x = fmaf(a.x, b.x, fmaf(a.y, b.y, f.x));
+                f.y = fmaf(a.x, b.y, fmaf(-a.y, b.x, f.y));
+            }
+            tot.x += (double)f.x;
+            tot.y += (double)f.y;
+        }
+    return tot;
+}
 template <int TS>
 struct G32Shape {
     static constexpr int NTH = TS * TS / 16, NG = 256 / NTH, RUNS = TS == 64 ? 4 : 2, KP = 8 * RUNS * NG;
@@ -261,91 +279,104 @@ __global__ void __launch_bounds__(256, 1) k_gram32(const float2 *__restrict__ ps
         }
         cp_async_commit();
     };
-    double2 tot[4][4];   // sums of the 4 x 4 entries
-    // PLAIN: every run added in FP64 by itself
-    auto sum_points = [&](auto plain) {
-        constexpr bool PLAIN = decltype(plain)::value;
-        float2 hi[4][4], lo[4][4];   // two-float sums of up to kGHeld runs, (re, im) pairs
+    // sums of the 4 x 4 entries: two-float sums of up to kGHeld runs, (re, im)
+    // pairs, and FP64
+    double2 tot[4][4];
+    float2 hi[4][4], lo[4][4];
 #pragma unroll
-        for (int i = 0; i < 4; i++)
+    for (int i = 0; i < 4; i++)
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                hi[i][j] = lo[i][j] = make_float2(0.f, 0.f);
-                tot[i][j] = make_double2(0.0, 0.0);
-            }
-        auto flush = [&]() {
+        for (int j = 0; j < 4; j++) {
+            hi[i][j] = lo[i][j] = make_float2(0.f, 0.f);
+            tot[i][j] = make_double2(0.0, 0.0);
+        }
+    // FP64 additions take 16 clocks a warp: the first flush has none to make
+    bool first = true;
+    auto flush = [&]() {
+        if (first) {
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    tot[i][j] = make_double2(widen(hi[i][j].x) + widen(lo[i][j].x), widen(hi[i][j].y) + widen(lo[i][j].y));
+        } else {
 #pragma unroll
             for (int i = 0; i < 4; i++)
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
                     tot[i][j].x += widen(hi[i][j].x) + widen(lo[i][j].x);
                     tot[i][j].y += widen(hi[i][j].y) + widen(lo[i][j].y);
-                    hi[i][j] = lo[i][j] = make_float2(0.f, 0.f);
                 }
-        };
-        if (p0 < p1) stage(p0, 0);
-        int k = 0, held = 0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) hi[i][j] = lo[i][j] = make_float2(0.f, 0.f);
+        first = false;
+    };
+    if (p0 < p1) stage(p0, 0);
+    int k = 0, held = 0;
+    for (int64_t pc = p0; pc < p1; pc += KP, k ^= 1) {
+        cp_async_wait<0>();
+        __syncthreads();
+        if (pc + KP < p1) stage(pc + KP, k ^ 1);
+        if (skip) continue;
+        const float2 *A = buf + k * BUFST + sr, *B = buf + k * BUFST + (TS == 64 && !diag ? G::PANEL : 0) + tc;
 #pragma unroll 1
-        for (int64_t pc = p0; pc < p1; pc += KP, k ^= 1) {
-            cp_async_wait<0>();
-            __syncthreads();
-            if (pc + KP < p1) stage(pc + KP, k ^ 1);
-            if (skip) continue;
-            const float2 *A = buf + k * BUFST + sr, *B = buf + k * BUFST + (TS == 64 && !diag ? G::PANEL : 0) + tc;
-#pragma unroll 1
-            for (int h = 0; h < G::RUNS; h++) {
-                float2 f[4][4];
+        for (int h = 0; h < G::RUNS; h++) {
+            float2 f[4][4];
 #pragma unroll
-                for (int i = 0; i < 4; i++)
+            for (int i = 0; i < 4; i++)
 #pragma unroll
-                    for (int j = 0; j < 4; j++) f[i][j] = make_float2(0.f, 0.f);
+                for (int j = 0; j < 4; j++) f[i][j] = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int q = 0; q < 8; q++) {
-                    const int row = ((g * G::RUNS + h) * 8 + q) * TS;
-                    const float4 a0 = *(const float4 *)(A + row), a1 = *(const float4 *)(A + row + 8);
-                    const float4 b0v = *(const float4 *)(B + row), b1v = *(const float4 *)(B + row + 2 * LX);
-                    const float2 x[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
-                                         make_float2(a1.z, a1.w)};
-                    const float2 y[4] = {make_float2(b0v.x, b0v.y), make_float2(b0v.z, b0v.w),
-                                         make_float2(b1v.x, b1v.y), make_float2(b1v.z, b1v.w)};
-#pragma unroll
-                    for (int i = 0; i < 4; i++)
-#pragma unroll
-                        for (int j = 0; j < 4; j++) {
-                            // conj(x) y
-                            f[i][j].x = fmaf(x[i].x, y[j].x, fmaf(x[i].y, y[j].y, f[i][j].x));
-                            f[i][j].y = fmaf(x[i].x, y[j].y, fmaf(-x[i].y, y[j].x, f[i][j].y));
-                        }
-                }
+            for (int q = 0; q < 8; q++) {
+                const int row = ((g * G::RUNS + h) * 8 + q) * TS;
+                const float4 a0 = *(const float4 *)(A + row), a1 = *(const float4 *)(A + row + 8);
+                const float4 b0v = *(const float4 *)(B + row), b1v = *(const float4 *)(B + row + 2 * LX);
+                const float2 x[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
+                                     make_float2(a1.z, a1.w)};
+                const float2 y[4] = {make_float2(b0v.x, b0v.y), make_float2(b0v.z, b0v.w), make_float2(b1v.x, b1v.y),
+                                     make_float2(b1v.z, b1v.w)};
 #pragma unroll
                 for (int i = 0; i < 4; i++)
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
-                        if constexpr (PLAIN) {
-                            tot[i][j].x += (double)f[i][j].x;
-                            tot[i][j].y += (double)f[i][j].y;
-                        } else {
-                            f2_two_sum(hi[i][j], lo[i][j], f[i][j]);
-                        }
+                        // conj(x) y
+                        f[i][j].x = fmaf(x[i].x, y[j].x, fmaf(x[i].y, y[j].y, f[i][j].x));
+                        f[i][j].y = fmaf(x[i].x, y[j].y, fmaf(-x[i].y, y[j].x, f[i][j].y));
                     }
             }
-            if (!PLAIN && (held += G::RUNS) >= kGHeld) {
-                flush();
-                held = 0;
-            }
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) f2_two_sum(hi[i][j], lo[i][j], f[i][j]);
         }
-        if (!PLAIN && !skip) flush();
-    };
-    sum_points(std::false_type{});
-    // runs that FP32 holds while their two-float sum does not
-    bool over = false;
+        if ((held += G::RUNS) >= kGHeld) {
+            flush();
+            held = 0;
+        }
+    }
+    if (held) flush();
+    auto row_of = [&](int i) { return sr + (i & 1) + 8 * (i >> 1); };
+    auto col_of = [&](int j) { return tc + (j & 1) + 2 * LX * (j >> 1); };
+    // sums that left the FP32 range: exponent of Inf and NaN
+    int top = 0;
 #pragma unroll
     for (int i = 0; i < 4; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) over = over || !isfinite(tot[i][j].x) || !isfinite(tot[i][j].y);
-    if (__syncthreads_or(over)) sum_points(std::true_type{});
-    auto row_of = [&](int i) { return sr + (i & 1) + 8 * (i >> 1); };
-    auto col_of = [&](int j) { return tc + (j & 1) + 2 * LX * (j >> 1); };
+        for (int j = 0; j < 4; j++)
+            top = max(top, max(__double2hiint(tot[i][j].x) & 0x7fffffff, __double2hiint(tot[i][j].y) & 0x7fffffff));
+    if (top >= 0x7ff00000) {
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int s = s0 + row_of(i), t = t0 + col_of(j);
+                if ((!isfinite(tot[i][j].x) || !isfinite(tot[i][j].y)) && s < S && t < S)
+                    tot[i][j] = gram_runs64(psi + s, psi + t, p0 + 8 * g * G::RUNS, p1, ld, G::RUNS, KP);
+            }
+    }
     if constexpr (G::NG == 1) {
         if (skip) return;
 #pragma unroll
